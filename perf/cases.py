@@ -183,7 +183,10 @@ def _batch_sets(case, seed):
     pair = torch.repeat_interleave(torch.arange(P, device="cuda").repeat_interleave(2), room, output_size=total)
     if case["data"] == "surface":
         axes = 0.2 + 0.8 * torch.rand(P, 3, device="cuda", generator=g)
-        q = torch.linalg.qr(torch.randn(P, 3, 3, device="cuda", generator=g))[0]
+        w, i, j, k = torch.nn.functional.normalize(torch.randn(P, 4, device="cuda", generator=g), dim=1).unbind(1)
+        q = torch.stack([1 - 2 * (j * j + k * k), 2 * (i * j - k * w), 2 * (i * k + j * w),
+                         2 * (i * j + k * w), 1 - 2 * (i * i + k * k), 2 * (j * k - i * w),
+                         2 * (i * k - j * w), 2 * (j * k + i * w), 1 - 2 * (i * i + j * j)], 1).reshape(P, 3, 3)
         box = torch.rand(P, device="cuda", generator=g) < 0.5
         ball = torch.nn.functional.normalize(torch.randn(total, 3, device="cuda", generator=g), dim=1)
         cube = torch.rand(total, 3, device="cuda", generator=g) * 2 - 1
