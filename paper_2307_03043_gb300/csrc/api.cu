@@ -65,11 +65,27 @@ struct Layout {
   }
 };
 
+// Where the workspace does not fit, the layout is taken again with the exact l2
+// scan in its CUDA-core form, which needs less scratch and gives the same bits.
 template <class F>
 static void carve(ch_ctx* c, F&& f) {
+  struct Restore {
+    ch_ctx* c;
+    bool was;
+    ~Restore() { c->exact_plain = was; }
+  } restore{c, c->exact_plain};
   Layout m;
   f(m);
-  c->ws.reserve(m.need + 256);
+  try {
+    c->ws.reserve(m.need + 256);
+  } catch (const Err& e) {
+    if (e.st != CH_ENOMEM || c->exact_plain) throw;
+    c->exact_plain = true;
+    Layout plain;
+    f(plain);
+    if (plain.need >= m.need) throw;
+    c->ws.reserve(plain.need + 256);
+  }
   c->ws.reset();
   Layout t;
   t.measure = false;
@@ -467,13 +483,30 @@ struct ScanBufs {
   ScanPart part;
   void* screen_work;
   int screen;
+  bool cert;  // the exact l2 scan runs in its certified tensor-core form
+  float* norms;  // its |b|^2 where the set's own cannot be used
 };
+
+// The exact l2 scan on c's stream can use the set's own |x|^2: the set belongs to c
+// (its lazy pass runs on c's stream, or c's parent's, which c's is ordered after) or
+// was prepared by a call that has returned.  Otherwise the scan makes its own: it
+// never wrote to another context's set, which others may be reading.
+static bool norms_usable(const ch_ctx* c, const ch_set* X) {
+  return X->ctx == c || X->ctx == c->parent || ((X->ready & READY_NORMS) && (X->ready & READY_SYNCED));
+}
 
 template <class L>
 static void take_scan(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, int64_t T, int metric, int screen,
-                      uint32_t R, ScanBufs* sb) {
+                      uint32_t R, ScanBufs* sb, bool plain = false) {
   sb->screen = screen_choice(screen, metric, A, B);
-  if (sb->screen == CH_SCREEN_EXACT) {
+  sb->cert = sb->screen == CH_SCREEN_EXACT && metric == CH_L2 && !plain && !c->exact_plain &&
+             exact_tc_supported(A, B, T);
+  if (sb->cert) {
+    sb->part = ScanPart{nullptr, nullptr, 0};
+    sb->screen_work =
+        lay.template take<char>(exact_tc_workspace(T, B->n, A->d, A->dtype, c->sm_count, c->screen_chunk_sms));
+    sb->norms = norms_usable(c, B) ? nullptr : lay.template take<float>(size_t(B->n));
+  } else if (sb->screen == CH_SCREEN_EXACT) {
     sb->part.chunks = scan_exact_chunks(T, B->n, A->d, A->dtype, c->sm_count);
     sb->part.val = lay.template take<float>(size_t(sb->part.chunks) * std::max<int64_t>(T, 1));
     sb->part.idx = lay.template take<int64_t>(size_t(sb->part.chunks) * std::max<int64_t>(T, 1));
@@ -490,7 +523,14 @@ static void run_scan(ch_ctx* c, const ch_set* A, const int64_t* idx, int64_t T, 
                      uint32_t R, ScanBufs* sb, float* m, int64_t* argmin, uint32_t* status,
                      const KernelTimer& timer = KernelTimer()) {
   if (T == 0) return;
-  if (sb->screen == CH_SCREEN_EXACT) {
+  if (sb->cert) {
+    timer.start(c->stream);
+    if (sb->norms) launch_norms(B, sb->norms, nullptr, c->stream);
+    else ensure_norms(const_cast<ch_set*>(B), c->stream);
+    launch_exact_tc(A, idx, T, B, sb->norms ? sb->norms : B->norms, sb->screen_work, m, argmin, c->sm_count,
+                    c->screen_chunk_sms, c->stream, c->wait_cycles);
+    timer.stop(c->stream);
+  } else if (sb->screen == CH_SCREEN_EXACT) {
     timer.start(c->stream);
     launch_scan_exact(A, idx, T, B, metric, sb->part, c->sm_count, c->stream);
     timer.stop(c->stream);
@@ -522,7 +562,7 @@ struct EstBufs {
 
 template <class L>
 static void take_estimate(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p, int64_t T,
-                          uint32_t R, EstBufs* eb) {
+                          uint32_t R, EstBufs* eb, bool plain = false) {
   const int64_t nA = A->n;
   eb->res = lay.template take<ResBlock>(1);
   eb->out2 = lay.template take<double>(kCombineDoubles);
@@ -534,16 +574,17 @@ static void take_estimate(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, c
   eb->w = lay.template take<uint64_t>(nA);
   eb->idx = lay.template take<int64_t>(std::max<int64_t>(T, 1));
   eb->m = lay.template take<float>(std::max<int64_t>(T, 1));
-  take_scan(lay, c, A, B, T, p->hash.metric, p->screen, R, &eb->sc);
+  take_scan(lay, c, A, B, T, p->hash.metric, p->screen, R, &eb->sc, plain);
 }
 
-// device workspace bytes ch_estimate(A, B, p) needs on a context like c
-size_t estimate_footprint(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p) {
+// device workspace bytes ch_estimate(A, B, p) needs on a context like c; with
+// plain, those of the CUDA-core form of the exact scan (what carve falls back to)
+size_t estimate_footprint(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p, bool plain) {
   const uint32_t R = p->rerank_k ? p->rerank_k : 8;
   const int64_t T = p->T > 0 ? p->T : default_T(A->n, B->n, p->eps);
   Layout m;
   EstBufs eb;
-  take_estimate(m, c, A, B, p, T, R, &eb);
+  take_estimate(m, c, A, B, p, T, R, &eb, plain);
   return m.need + 256;
 }
 
@@ -767,6 +808,7 @@ ch_status ch_set_embed(ch_ctx* c, ch_set* X, const ch_hash_params* hp) {
   launch_k(k_collect, 1, 32, 0, s, res, X->status, nullptr, nullptr, nullptr, nullptr, nullptr);
   launch_check("collect");
   finish(c, res, static_cast<ResBlock*>(c->host_pin));
+  X->ready |= READY_SYNCED;
   X->hs.seed = hp->hash_seed;
   X->hs.k = k;
   X->hs.valid = true;
@@ -788,6 +830,7 @@ ch_status ch_set_prepare(ch_ctx* c, ch_set* X) {
   launch_k(k_collect, 1, 32, 0, s, res, X->status, nullptr, nullptr, nullptr, nullptr, nullptr);
   launch_check("collect");
   finish(c, res, static_cast<ResBlock*>(c->host_pin));
+  X->ready |= READY_SYNCED;
   return CH_OK;
   CHX_GUARD_END
 }
@@ -1408,6 +1451,7 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
     ch_ctx* l = nullptr;
     const ch_status cs = ch_ctx_create(c->device, nullptr, &l);
     CHX_CHECK(cs == CH_OK, cs, "batch lane creation failed");
+    l->parent = c;
     c->lanes.push_back(l);
   }
   // K lanes run at once, so each screen splits B for its share of the SMs only
@@ -1446,21 +1490,32 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
   std::vector<char> bcr(count, 0);
   for (int64_t i : run) bcr[i] = crude_batchable(A[i], B[i], &params[i]);
   std::vector<size_t> need(K, 0);
-  for (int64_t i : run) {
-    const ch_est_params* p = &params[i];
-    ch_ctx* lane = c->lanes[i % K];
-    Layout mc, ms;
-    CrudeBufs cb;
-    if (!bcr[i]) {
-      take_crude(mc, A[i], B[i], &p->hash, &cb);
-      mc.template take<int64_t>(A[i]->n);  // b(a)
-      mc.template take<uint8_t>(A[i]->n);  // level
+  auto lane_needs = [&] {
+    std::fill(need.begin(), need.end(), 0);
+    for (int64_t i : run) {
+      const ch_est_params* p = &params[i];
+      ch_ctx* lane = c->lanes[i % K];
+      Layout mc, ms;
+      CrudeBufs cb;
+      if (!bcr[i]) {
+        take_crude(mc, A[i], B[i], &p->hash, &cb);
+        mc.template take<int64_t>(A[i]->n);  // b(a)
+        mc.template take<uint8_t>(A[i]->n);  // level
+      }
+      ScanBufs sc;
+      if (!small[i]) take_scan(ms, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc);
+      need[i % K] = std::max(need[i % K], std::max(mc.need, ms.need) + 256);
     }
-    ScanBufs sc;
-    if (!small[i]) take_scan(ms, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc);
-    need[i % K] = std::max(need[i % K], std::max(mc.need, ms.need) + 256);
+    for (int k = 0; k < K; ++k) c->lanes[k]->ws.reserve(need[k]);
+  };
+  for (int k = 0; k < K; ++k) c->lanes[k]->exact_plain = false;
+  try {
+    lane_needs();
+  } catch (const Err& e) {  // the exact l2 scans' CUDA-core form needs less scratch (see carve)
+    if (e.st != CH_ENOMEM) throw;
+    for (int k = 0; k < K; ++k) c->lanes[k]->exact_plain = true;
+    lane_needs();
   }
-  for (int k = 0; k < K; ++k) c->lanes[k]->ws.reserve(need[k]);
   // the batch allocation: result blocks, the work list, then each pair's arrays
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   size_t arena = al(sizeof(ResBlock) * count) + al(sizeof(BatchItem) * std::max<size_t>(run.size(), 1));

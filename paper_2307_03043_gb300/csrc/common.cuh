@@ -128,6 +128,7 @@ struct ch_ctx {
   bool own_stream = false;
   int sm_count = 0;
   int screen_chunk_sms = 0;  // SMs the screen's B split aims to fill (0: all); a batch lane's share
+  bool exact_plain = false;  // the exact l2 scan keeps to CUDA cores (a call whose certified form's scratch did not fit)
   long long wait_cycles = 0;  // budget of the tensor-core screen's pipeline waits, SM cycles (0: about 2 s)
   chx::Arena ws;
   cudaMemPool_t pool = nullptr;  // stream-ordered pool for sets; keeps freed memory
@@ -135,6 +136,7 @@ struct ch_ctx {
   std::string err;
   cudaEvent_t ev[8] = {};
   std::vector<ch_ctx*> lanes;  // sub-contexts (own streams) of batched calls, made on first use
+  ch_ctx* parent = nullptr;    // the context a batch lane belongs to
   cudaStream_t side = nullptr;  // second stream for work that runs beside the main one, made on first use
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   void* batch_pin = nullptr;   // pinned result blocks of batched calls
@@ -160,11 +162,14 @@ namespace chx {
 enum : uint32_t {
   READY_BOX_X = 1u << 0,  // box_x computed (and the finite check done)
   READY_NORMS = 1u << 1,  // norms computed (and the finite check done)
+  READY_SYNCED = 1u << 2,  // the passes above have finished on the device (ch_set_prepare, ch_set_embed)
 };
 // ingest pass (box of x, finite check) unless already done
 void ensure_ingest(ch_set* X, cudaStream_t s);
 // |x|^2 per row (sequential fmaf chain over j) unless already done
 void ensure_norms(ch_set* X, cudaStream_t s);
+// the same into norms [n]; status: raised for a non-finite value, or null
+void launch_norms(const ch_set* X, float* norms, uint32_t* status, cudaStream_t s);
 }  // namespace chx
 
 namespace chx {
@@ -540,6 +545,36 @@ size_t screen_workspace(int64_t T, int64_t nB, int d, int R, int sm_count, int c
 void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int screen, int R,
                       void* work, float* min_d, int64_t* argmin, uint32_t* status, int sm_count, int chunk_sms,
                       cudaStream_t s, const KernelTimer& timer, long long wait_cycles = 0);
+
+// Certified exact l2 scan (k_screen.cu): the tensor-core screen with a proven
+// error bound picks the columns whose canonical distance is evaluated; min_d and
+// argmin are the exact scan's, bit for bit.
+bool exact_tc_supported(const ch_set* A, const ch_set* B, int64_t T);
+size_t exact_tc_workspace(int64_t T, int64_t nB, int d, int dtype, int sm_count, int chunk_sms);
+void launch_exact_tc(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const float* normB, void* work,
+                     float* min_d, int64_t* argmin, int sm_count, int chunk_sms, cudaStream_t s, long long wait_cycles);
+
+// k_certify's part of it: samples l0 .. l0 + T - 1 with their screened classes
+// (part_* [parts][T][32]; part p covers chunk p / slices of B, columns
+// t * tile + (p % slices) * 128 + o * 32 + class, o < 4, of its tiles t)
+struct CertArgs {
+  int64_t l0, T, nB, chunk_len;
+  int d, parts, slices, tile;
+  const float* part_s;
+  const int32_t* part_i;
+  const float* part_2;
+  double p_scale, q_scale;  // a column is evaluated when L <= P p_scale - |q|^2 q_scale + 2^-100
+  int64_t limit;            // most columns evaluated per sample
+  int32_t* list;            // samples left to k_scan_exact's list form
+  uint32_t* ctl;            // [0] their number, [1] set when a screen gave up
+  unsigned long long* best; // [T of the call] the list form's minima, set to all ones with each listing
+};
+void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, const CertArgs& c, float* min_d,
+                    int64_t* argmin, cudaStream_t s);
+// the exact scan of the ctl[0] listed samples (at most T), written to their places
+void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const int32_t* list,
+                      const uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,
+                      cudaStream_t s);
 
 // result block copied to the host at the end of a synchronising call
 struct ResBlock {

@@ -126,37 +126,93 @@ void ensure_ingest(ch_set* X, cudaStream_t s) {
   X->ready |= READY_BOX_X;
 }
 
-// |x|^2 per row as the fmaf chain over j in increasing order (the order the l2
-// projection pass uses, so the norms never depend on which pass made them)
+// the coordinates of a 16-byte word of a row (FP8: times the row's scale)
 template <int DT>
-__global__ void __launch_bounds__(256) k_norms(const void* X, const float* scales, int64_t n, int d, float* norms,
-                                               uint32_t* status) {
+__device__ __forceinline__ void chunk_vals(const uint4 raw, float sc, float (&v)[16 / (DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1)]) {
+  if constexpr (DT == CH_F32) {
+    v[0] = __uint_as_float(raw.x);
+    v[1] = __uint_as_float(raw.y);
+    v[2] = __uint_as_float(raw.z);
+    v[3] = __uint_as_float(raw.w);
+  } else if constexpr (DT == CH_BF16) {
+    const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      v[2 * e] = __uint_as_float(w4[e] << 16);
+      v[2 * e + 1] = __uint_as_float(w4[e] & 0xFFFF0000u);
+    }
+  } else {
+    const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+    for (int e = 0; e < 16; ++e) v[e] = __fmul_rn(e4m3_to_f32(static_cast<uint8_t>(w4[e / 4] >> (8 * (e % 4)))), sc);
+  }
+}
+
+// |x|^2 per row as the fmaf chain over j in increasing order (the order the l2
+// projection pass uses, so the norms never depend on which pass made them).  A
+// thread per row; VEC (rows of a multiple of 16 bytes on 16-byte aligned bases)
+// reads them in 16-byte words, so a warp's 32 row segments stay in L1 for the words
+// that follow, and blocks of 64 threads spread small sets over the SMs.
+template <int DT, bool VEC>
+__global__ void __launch_bounds__(64) k_norms(const void* X, const float* scales, int64_t n, int d, float* norms,
+                                              uint32_t* status) {
   pdl_entry();
   const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   bool bad = false;
   if (r < n) {
     float sq = 0.0f;
-    for (int j = 0; j < d; ++j) {
-      const float x = load_elem<DT>(X, r, d, j, scales);
-      bad |= !isfinite(x);
-      sq = fmaf(x, x, sq);
+    if constexpr (VEC) {
+      constexpr int PER = 16 / (DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1);
+      const int words = d / PER;
+      const uint4* row = static_cast<const uint4*>(X) + r * words;
+      const float sc = DT == CH_FP8E4M3 ? scales[r] : 1.0f;
+      constexpr int U = 8;
+      for (int m0 = 0; m0 < words; m0 += U) {
+        uint4 w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (m0 + u < words) w[u] = row[m0 + u];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (m0 + u < words) {
+            float v[PER];
+            chunk_vals<DT>(w[u], sc, v);
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+              bad |= !isfinite(v[e]);
+              sq = fmaf(v[e], v[e], sq);
+            }
+          }
+      }
+    } else {
+      for (int j = 0; j < d; ++j) {
+        const float x = load_elem<DT>(X, r, d, j, scales);
+        bad |= !isfinite(x);
+        sq = fmaf(x, x, sq);
+      }
     }
     norms[r] = sq;
   }
-  if (__any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_NONFINITE);
+  if (status && __any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_NONFINITE);
+}
+
+void launch_norms(const ch_set* X, float* norms, uint32_t* status, cudaStream_t s) {
+  if (X->n == 0) return;
+  const int grid = static_cast<int>(ceil_div(X->n, 64));
+  const bool vec = (size_t(X->d) * elem_size(X->dtype)) % 16 == 0 && (reinterpret_cast<uintptr_t>(X->data) & 15) == 0;
+  auto go = [&](auto kern) { launch_k(kern, grid, 64, 0, s, X->data, X->scales, X->n, X->d, norms, status); };
+  switch (X->dtype) {
+    case CH_F32: vec ? go(k_norms<CH_F32, true>) : go(k_norms<CH_F32, false>); break;
+    case CH_BF16: vec ? go(k_norms<CH_BF16, true>) : go(k_norms<CH_BF16, false>); break;
+    default: vec ? go(k_norms<CH_FP8E4M3, true>) : go(k_norms<CH_FP8E4M3, false>); break;
+  }
+  launch_check("norms");
 }
 
 void ensure_norms(ch_set* X, cudaStream_t s) {
   if (X->ready & READY_NORMS) return;
   X->ready |= READY_NORMS;
-  if (X->n == 0) return;
-  const int grid = static_cast<int>(ceil_div(X->n, 256));
-  switch (X->dtype) {
-    case CH_F32: launch_k(k_norms<CH_F32>, grid, 256, 0, s, X->data, X->scales, X->n, X->d, X->norms, X->status); break;
-    case CH_BF16: launch_k(k_norms<CH_BF16>, grid, 256, 0, s, X->data, X->scales, X->n, X->d, X->norms, X->status); break;
-    default: launch_k(k_norms<CH_FP8E4M3>, grid, 256, 0, s, X->data, X->scales, X->n, X->d, X->norms, X->status); break;
-  }
-  launch_check("norms");
+  launch_norms(X, X->norms, X->status, s);
 }
 
 // ------------------------------------------------------------------ l2 embedding
@@ -1254,27 +1310,6 @@ void launch_crude_dist_batch(const CrudePair* P, const int* blk0, int np, int bl
 // increasing j.  The tree p_q += p_{q+s} for s = 16 .. 1 runs by shuffles inside
 // the group for s >= C and in registers below: the same sums, in the same order,
 // as the lane-per-partial form.
-template <int DT>
-__device__ __forceinline__ void chunk_vals(const uint4 raw, float sc, float (&v)[16 / (DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1)]) {
-  if constexpr (DT == CH_F32) {
-    v[0] = __uint_as_float(raw.x);
-    v[1] = __uint_as_float(raw.y);
-    v[2] = __uint_as_float(raw.z);
-    v[3] = __uint_as_float(raw.w);
-  } else if constexpr (DT == CH_BF16) {
-    const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      v[2 * e] = __uint_as_float(w4[e] << 16);
-      v[2 * e + 1] = __uint_as_float(w4[e] & 0xFFFF0000u);
-    }
-  } else {
-    const uint32_t w4[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-    for (int e = 0; e < 16; ++e) v[e] = __fmul_rn(e4m3_to_f32(static_cast<uint8_t>(w4[e / 4] >> (8 * (e % 4)))), sc);
-  }
-}
-
 // Resident blocks of the vector crude-distance kernel per SM.  Each lane keeps
 // all its chunks of a and of b(a) in flight at once (d / 32 of each: 12 at d =
 // 384), and the row group's b(a) is read one row group ahead, so a row costs

@@ -145,12 +145,32 @@ __device__ __forceinline__ void stage_row_async(float* __restrict__ Ts, int r, c
 // One block: QT samples against a chunk of B, staged SUB x BT rows at a time
 // (one pair of barriers per stage); each thread owns PQ samples x PB rows of
 // every BT-row sub-tile.
-template <int DT, int METRIC, int QT, int BT, int PQ, int PB, int NJ, int SUB, bool DB>
+// LIST (what the certified scan leaves over): the samples are the *count listed
+// ones, known only on the device, so a persistent grid cuts B into as many chunks
+// as keep its blocks busy for that count (none listed: every block returns), and
+// the minima fold into best[] as (distance bits, index) words by atomicMin.
+struct ScanList {
+  const int32_t* list;
+  const uint32_t* count;
+  unsigned long long* best;
+};
+
+template <int DT, int METRIC, int QT, int BT, int PQ, int PB, int NJ, int SUB, bool DB, bool LIST>
 __global__ void __launch_bounds__(256, kScanBlocksPerSM)
     k_scan_exact(const void* __restrict__ A, const float* __restrict__ scA, const int64_t* __restrict__ qidx, int64_t T,
                  int64_t nA, const void* __restrict__ B, const float* __restrict__ scB, int64_t nB, int d,
-                 int64_t chunk_len, float* part_val, int64_t* part_idx) {
+                 int64_t chunk_len, float* part_val, int64_t* part_idx, ScanList sl) {
   pdl_entry();
+  int64_t qtiles = 1, items = 1;
+  if constexpr (LIST) {
+    T = *sl.count;
+    if (T == 0) return;
+    qtiles = (T + QT - 1) / QT;
+    const int64_t stages = (nB + BT * SUB - 1) / (BT * SUB);
+    const int64_t want = max(int64_t(1), min((stages + 3) / 4, (4 * int64_t(gridDim.x) + qtiles - 1) / qtiles));
+    chunk_len = (stages + want - 1) / want * (BT * SUB);
+    items = qtiles * ((nB + chunk_len - 1) / chunk_len);
+  }
   constexpr int NTQ = QT / PQ, NTB = BT / PB;
   static_assert(NTQ * NTB == 256, "256 threads");
   static_assert(NTB == 16, "16 thread rows (the occupancy estimate assumes it)");
@@ -164,16 +184,18 @@ __global__ void __launch_bounds__(256, kScanBlocksPerSM)
 
   const int tid = threadIdx.x;
   const int tq = tid % NTQ, tb = tid / NTQ;
-  const int64_t q0 = int64_t(blockIdx.x) * QT;
-  const int64_t b_begin = int64_t(blockIdx.y) * chunk_len;
+  for (int64_t item = LIST ? int64_t(blockIdx.x) : 0; item < items; item += gridDim.x) {
+  const int64_t q0 = (LIST ? item % qtiles : int64_t(blockIdx.x)) * QT;
+  const int64_t b_begin = (LIST ? item / qtiles : int64_t(blockIdx.y)) * chunk_len;
   const int64_t b_end = min(nB, b_begin + chunk_len);
 
   // tiles are staged transposed (coordinate-major), four rows per warp instruction
   const int warp = tid >> 5, rl = (tid & 31) & 3, jl = (tid & 31) >> 2;
   for (int g = warp; g < QT / 4; g += 8) {
     const int q = 4 * g + rl;
-    const int64_t l = q0 + q;
-    int64_t a = l < T ? (qidx ? qidx[l] : l) : -1;
+    int64_t l = q0 + q;
+    if constexpr (LIST) l = l < T ? int64_t(sl.list[l]) : INT64_MAX;
+    int64_t a = (LIST ? l != INT64_MAX : l < T) ? (qidx ? qidx[l] : l) : -1;
     if (a >= nA) a = -1;
     stage_row<DT, QS, NJ>(Qs, q, A, scA, a, d, jl);
   }
@@ -273,10 +295,27 @@ __global__ void __launch_bounds__(256, kScanBlocksPerSM)
       }
     }
     const int64_t l = q0 + tid;
-    if (l < T) {
+    if constexpr (LIST) {
+      if (l < T && bi != INT64_MAX)
+        atomicMin(&sl.best[l], (static_cast<unsigned long long>(__float_as_uint(bv)) << 32) | static_cast<uint32_t>(bi));
+    } else if (l < T) {
       part_val[int64_t(blockIdx.y) * T + l] = bv;
       part_idx[int64_t(blockIdx.y) * T + l] = bi;
     }
+  }
+  if constexpr (LIST) __syncthreads();  // the tiles and minima are rewritten by the next item
+  }
+}
+
+// the listed samples' minima to their places
+__global__ void k_scan_list_out(ScanList sl, float* min_d, int64_t* argmin) {
+  pdl_entry();
+  const int64_t n = *sl.count;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
+    const unsigned long long v = sl.best[i];
+    const int64_t l = sl.list[i];
+    min_d[l] = v == ~0ull ? __int_as_float(0x7F800000) : __uint_as_float(static_cast<uint32_t>(v >> 32));
+    if (argmin) argmin[l] = v == ~0ull ? INT64_MAX : static_cast<int64_t>(v & 0xFFFFFFFFull);
   }
 }
 
@@ -521,37 +560,46 @@ int scan_exact_chunks(int64_t T, int64_t nB, int d, int dtype, int sm_count) {
 
 template <int DT, int METRIC, int QT, int BT, int PQ, int PB, int NJ = 0, int SUB = 1>
 static void scan_launch(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, ScanPart part,
-                        cudaStream_t s) {
+                        cudaStream_t s, const ScanList& list) {
   constexpr bool kDB = DT == CH_F32 && NJ > 0 && NJ <= 2;  // the launches of scan_double_buffered(DT, d)
-  auto kern = k_scan_exact<DT, METRIC, QT, BT, PQ, PB, NJ, SUB, kDB>;
   const bool db = kDB;
   CHX_CHECK(tile_for(A->d).BT == BT && tile_for(A->d).SUB == SUB, CH_ENOTSUP, "scan tile mismatch");
   const size_t smem = scan_smem(A->d, db);
+  if (list.list) {
+    if constexpr (METRIC == CH_L2 && DT != CH_FP8E4M3) {
+      auto kern = k_scan_exact<DT, METRIC, QT, BT, PQ, PB, NJ, SUB, kDB, true>;
+      CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+      launch_k(kern, part.chunks * scan_blocks_per_sm(A->d, db), 256, smem, s, A->data, A->scales, qidx, T, A->n,
+               B->data, B->scales, B->n, A->d, int64_t(0), part.val, part.idx, list);
+    }
+    return;
+  }
   // a constant value, so concurrent callers on other threads never race on it
+  auto kern = k_scan_exact<DT, METRIC, QT, BT, PQ, PB, NJ, SUB, kDB, false>;
   CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   const int64_t chunk_len = ceil_div(ceil_div(B->n, part.chunks), BT * SUB) * (BT * SUB);
   dim3 grid(static_cast<unsigned>(ceil_div(T, QT)), static_cast<unsigned>(part.chunks));
   launch_k(kern, grid, 256, smem, s, A->data, A->scales, qidx, T, A->n, B->data, B->scales, B->n, A->d, chunk_len,
-                               part.val, part.idx);
+           part.val, part.idx, list);
 }
 
 template <int DT, int METRIC>
 static void scan_shape(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, ScanPart part,
-                       cudaStream_t s) {
+                       cudaStream_t s, const ScanList& list = ScanList{nullptr, nullptr, nullptr}) {
   const TileShape t = tile_for(A->d);
   if (A->d <= 128) {  // terms per partial fixed at compile time
     switch ((A->d + 31) / 32) {
-      case 1: scan_launch<DT, METRIC, 32, 64, 2, 4, 1, 4>(A, qidx, T, B, part, s); break;
-      case 2: scan_launch<DT, METRIC, 32, 64, 2, 4, 2>(A, qidx, T, B, part, s); break;
-      case 3: scan_launch<DT, METRIC, 32, 64, 2, 4, 3>(A, qidx, T, B, part, s); break;
-      default: scan_launch<DT, METRIC, 32, 64, 2, 4, 4>(A, qidx, T, B, part, s); break;
+      case 1: scan_launch<DT, METRIC, 32, 64, 2, 4, 1, 4>(A, qidx, T, B, part, s, list); break;
+      case 2: scan_launch<DT, METRIC, 32, 64, 2, 4, 2>(A, qidx, T, B, part, s, list); break;
+      case 3: scan_launch<DT, METRIC, 32, 64, 2, 4, 3>(A, qidx, T, B, part, s, list); break;
+      default: scan_launch<DT, METRIC, 32, 64, 2, 4, 4>(A, qidx, T, B, part, s, list); break;
     }
   } else if (t.BT == 64)
-    scan_launch<DT, METRIC, 32, 64, 2, 4>(A, qidx, T, B, part, s);
+    scan_launch<DT, METRIC, 32, 64, 2, 4>(A, qidx, T, B, part, s, list);
   else if (t.BT == 32)
-    scan_launch<DT, METRIC, 32, 32, 2, 2>(A, qidx, T, B, part, s);
+    scan_launch<DT, METRIC, 32, 32, 2, 2>(A, qidx, T, B, part, s, list);
   else
-    scan_launch<DT, METRIC, 16, 16, 1, 1>(A, qidx, T, B, part, s);
+    scan_launch<DT, METRIC, 16, 16, 1, 1>(A, qidx, T, B, part, s, list);
 }
 
 template <int DT, int METRIC, int D>
@@ -608,6 +656,22 @@ void launch_scan_merge(ScanPart part, int64_t T, const int64_t* qidx, float* min
   launch_k(k_scan_merge, static_cast<int>(ceil_div(T, 256)), 256, 0, s, part.val, part.idx, part.chunks, T, qidx, min_d,
                                                                   argmin);
   launch_check("scan_merge");
+}
+
+void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const int32_t* list,
+                      const uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,
+                      cudaStream_t s) {
+  CHX_CHECK(scan_smem(A->d, false) <= 220 * 1024, CH_ENOTSUP, "dimension too large for the exact scan");
+  const ScanList sl{list, ctl, best};
+  const ScanPart grid{nullptr, nullptr, sm_count};  // the list form's grid: sm_count x resident blocks
+  if (A->dtype == CH_F32)
+    scan_shape<CH_F32, CH_L2>(A, qidx, T, B, grid, s, sl);
+  else
+    scan_shape<CH_BF16, CH_L2>(A, qidx, T, B, grid, s, sl);
+  launch_check("scan_list");
+  launch_k(k_scan_list_out, static_cast<int>(std::min<int64_t>(ceil_div(T, 256), sm_count)), 256, 0, s, sl, min_d,
+           argmin);
+  launch_check("scan_list_out");
 }
 
 int small_scan_samples_per_item() { return kBatchQ; }

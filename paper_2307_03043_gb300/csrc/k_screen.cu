@@ -145,6 +145,7 @@ struct ScreenArgs {
   int64_t T;          // samples (rows of Q)
   int64_t nB;
   int kblocks;        // ceil(d * elem / 128)
+  int last_steps;     // 32-byte steps of the last K block that hold coordinates
   int row_tiles;
   int chunks;
   int64_t chunk_len;  // B points per chunk (multiple of kBN)
@@ -153,9 +154,12 @@ struct ScreenArgs {
   const float* normB;   // |b|^2 [nB]
   const float* scaleB;  // FP8 row scales [nB] or null
   const float* scaleQ;  // FP8 sample scales [T] or null
-  float* part_s;        // [chunks][T][R]
+  float* part_s;        // [chunks * kSlices][T][kClasses]
   int32_t* part_i;
-  uint32_t* status;
+  float* part_2;        // certified form: the classes' second-smallest tile minima, same layout
+  float shrink;         // certified form: factor of |b|^2 that makes a score a lower bound
+  uint32_t* status;     // receives fail_bit if a pipeline wait ran out
+  uint32_t fail_bit;
   long long wait_cycles;  // budget of each pipeline wait (SM cycles)
 };
 
@@ -172,7 +176,11 @@ __device__ __forceinline__ void mbar_arrive_relaxed(uint32_t addr) {
 // item `item` covers sample tile tile_of(item) and chunk item / items_per_chunk.
 // After reading an accumulator each warp arrives once on acc_empty[acc] (given by
 // its shared address).
-template <int SCREEN, class TileOf>
+// CERT (the certified exact scan): |b|^2 is scaled by args.shrink (rounded down)
+// as it is staged, so that a score plus the sample's share is a lower bound of the
+// distance, and each class also keeps its second-smallest tile minimum: whatever
+// lies in the class outside the kept tile scored at least that.
+template <int SCREEN, bool CERT, class TileOf>
 __device__ __forceinline__ void screen_epilogue(const ScreenArgs& args, int first_item, int item_stride, int n_items,
                                               int items_per_chunk, TileOf tile_of, uint32_t tmem_base,
                                               float* nb_s, float* sb_s, uint64_t* acc_full,
@@ -195,10 +203,12 @@ __device__ __forceinline__ void screen_epilogue(const ScreenArgs& args, int firs
     // running minima per residue class of this warp's slice; best_c holds the
     // tile (within the chunk) of each minimum
     float best_s[kClasses];
+    float next_s[CERT ? kClasses : 1];
     int32_t best_c[kClasses];
 #pragma unroll
     for (int i = 0; i < kClasses; ++i) {
       best_s[i] = __int_as_float(0x7F800000);
+      if constexpr (CERT) next_s[i] = __int_as_float(0x7F800000);
       best_c[i] = -1;
     }
     int32_t tile = 0;  // tile index within the chunk
@@ -213,6 +223,7 @@ __device__ __forceinline__ void screen_epilogue(const ScreenArgs& args, int firs
       for (int k = 0; k < kPer; ++k) {
         const int64_t b = base + lane + 32 * k;
         pn[k] = (b < b_end) ? __ldg(&args.normB[b]) : __int_as_float(0x7F800000);
+        if constexpr (CERT) pn[k] = __fmul_rd(pn[k], args.shrink);
         ps[k] = 0.0f;
         if constexpr (SCREEN == CH_SCREEN_FP8) ps[k] = (b < b_end) ? -2.0f * __ldg(&args.scaleB[b]) : 0.0f;
       }
@@ -280,6 +291,7 @@ __device__ __forceinline__ void screen_epilogue(const ScreenArgs& args, int firs
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           const bool lt = tm[i] < best_s[h + i];
+          if constexpr (CERT) next_s[h + i] = fminf(next_s[h + i], fmaxf(best_s[h + i], tm[i]));
           best_s[h + i] = lt ? tm[i] : best_s[h + i];
           best_c[h + i] = lt ? tile : best_c[h + i];
         }
@@ -324,18 +336,23 @@ __device__ __forceinline__ void screen_epilogue(const ScreenArgs& args, int firs
       // entry (tile t, class i) stands for columns
       // b_begin + t*256 + slice*kSliceCols + o*kClasses + i, o = 0 .. kOcc-1
       const size_t base = (size_t(ck * kSlices + qs) * args.T + grow) * kClasses;
+      const int32_t c0 = static_cast<int32_t>(b_begin) + qs * kSliceCols;
+      auto first_col = [&](int i) { return best_c[i] < 0 ? -1 : c0 + best_c[i] * kBN + i; };
 #pragma unroll
-      for (int i = 0; i < kClasses; ++i) {
-        const int32_t t = best_c[i];
-        args.part_s[base + i] = best_s[i];
-        args.part_i[base + i] =
-            t < 0 ? -1 : static_cast<int32_t>(b_begin + int64_t(t) * kBN + qs * kSliceCols + i);
+      for (int i = 0; i < kClasses; i += 4) {  // 16-byte stores: a row's 32 entries are one 128-byte line
+        *reinterpret_cast<float4*>(args.part_s + base + i) =
+            make_float4(best_s[i], best_s[i + 1], best_s[i + 2], best_s[i + 3]);
+        *reinterpret_cast<int4*>(args.part_i + base + i) =
+            make_int4(first_col(i), first_col(i + 1), first_col(i + 2), first_col(i + 3));
+        if constexpr (CERT)
+          *reinterpret_cast<float4*>(args.part_2 + base + i) =
+              make_float4(next_s[i], next_s[i + 1], next_s[i + 2], next_s[i + 3]);
       }
     }
   }
   }
 
-template <int SCREEN, bool STREAMQ>
+template <int SCREEN, bool STREAMQ, bool CERT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_screen(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmB, ScreenArgs args) {
   pdl_entry();
@@ -469,9 +486,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const uint32_t qa = su32(q_smem + size_t(streamq ? stage : kb) * kBM * kKB);
             const uint32_t ba = su32(b_smem + size_t(stage) * kBN * kKB);
+            // 32 bytes of K per instruction; the last K block's zero tail is left out
+            const int steps = kb + 1 < KB ? kKB / 32 : args.last_steps;
 #pragma unroll
-            for (int k = 0; k < kKB / 32; ++k)  // 32 bytes of K per instruction
-              tc_mma<SCREEN>(dtmem, sdesc(qa + k * 32), sdesc(ba + k * 32), (kb > 0 || k > 0) ? 1u : 0u);
+            for (int k = 0; k < kKB / 32; ++k)
+              if (k < steps) tc_mma<SCREEN>(dtmem, sdesc(qa + k * 32), sdesc(ba + k * 32), (kb > 0 || k > 0) ? 1u : 0u);
             tc_commit(&empty[stage]);
             if (++stage == S) {
               stage = 0;
@@ -492,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     uint32_t acc_empty_c[2] = {su32(&acc_empty[0]), su32(&acc_empty[1])};
-    screen_epilogue<SCREEN>(args, blockIdx.x, gridDim.x, n_items, args.row_tiles,
+    screen_epilogue<SCREEN, CERT>(args, blockIdx.x, gridDim.x, n_items, args.row_tiles,
                             [&](int item) { return item % args.row_tiles; }, tmem_base, nb_s, sb_s, acc_full,
                             acc_empty_c, abort_flag, budget);
   }
@@ -500,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // ------------------------------------------------ teardown
   // (the producer and the MMA thread have drained their copies and MMAs above)
   __syncwarp();
-  if (*abort_flag && threadIdx.x == 0) atomicOr(args.status, ST_TIMEOUT);
+  if (*abort_flag && threadIdx.x == 0) atomicOr(args.status, args.fail_bit);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -550,6 +569,9 @@ struct Plan {
   size_t smem;
   int grid;
 };
+
+// 32-byte MMA steps that cover the last 128-byte K block of a row
+int last_steps_of(int row_bytes) { return static_cast<int>(ceil_div(row_bytes - (ceil_div(row_bytes, kKB) - 1) * kKB, 32)); }
 
 int screen_dtype(int screen) { return screen == CH_SCREEN_TF32 ? CH_F32 : screen == CH_SCREEN_BF16 ? CH_BF16 : CH_FP8E4M3; }
 
@@ -655,6 +677,7 @@ void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
   a.T = T;
   a.nB = B->n;
   a.kblocks = p.kblocks;
+  a.last_steps = last_steps_of(row_bytes);
   a.row_tiles = p.row_tiles;
   a.chunks = p.chunks;
   a.chunk_len = p.chunk_len;
@@ -665,12 +688,15 @@ void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
   a.scaleQ = sQ;
   a.part_s = part_s;
   a.part_i = part_i;
+  a.part_2 = nullptr;
+  a.shrink = 1.0f;
   a.status = status;
+  a.fail_bit = ST_TIMEOUT;
   a.wait_cycles = wait_cycles > 0 ? wait_cycles : kTimeoutCycles;
 
 #define CHX_SCREEN_LAUNCH(SCR)                                                                              \
   do {                                                                                                      \
-    auto kern = p.stream_q ? k_screen<SCR, true> : k_screen<SCR, false>;                                    \
+    auto kern = p.stream_q ? k_screen<SCR, true, false> : k_screen<SCR, false, false>;                                 \
     CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)); /* constant */ \
     timer.start(s);                                                                                         \
     launch_k(kern, p.grid, kThreads, p.smem, s, tmQ, tmB, a);                                               \
@@ -683,6 +709,146 @@ void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
   launch_check("screen");
 
   launch_rerank(A, qidx, T, B, part_s, part_i, kSlices * p.chunks, kClasses, kOcc, kClasses, p.R, min_d, argmin, s);
+}
+
+// ------------------------------------------------------------------ certified exact scan
+// The exact l2 scan through the same contraction: the screen's scores only decide
+// which columns are evaluated, and a proven bound on their error decides it, so the
+// minimum and argmin are those of the canonical distance to every b, bit for bit.
+//
+// For real D2 = |q - b|^2 and the computed score S = fl(|b|^2 - 2 acc):
+//   |S + |q|^2 - D2| <= a |q||b| + b1 |b|^2,
+//   a  = 2 (c_in + 4 d 2^-23) + 2^-22: operand rounding (binary32 rows read as tf32
+//        keep 10 mantissa bits: c_in = 2^-9 (1 + 2^-10) per product for truncation or
+//        rounding; bf16 products are exact), accumulation (each of the d products is
+//        added with an error of at most 2^-23 of the largest partial sum, times four
+//        for margin; the partial sums are at most |q||b|), and the last fma;
+//   b1 = (d + 2) 2^-23: the norm's fma chain and the last fma.
+// With |q||b| <= (|q|^2 + |b|^2) / 2 the two sides separate:
+//   D2 >= L(b) + |q|^2 (1 - a/2),  L(b) = fl(|b|^2 (1 - a/2 - b1) - 2 acc)
+// so a point far from everything cannot widen the bound of the others.  A canonical
+// squared distance P is within g D2 of D2, g = (ceil(d/32) + 9) 2^-24, and square
+// roots of values within 2^-22 of one another may round to the same distance, so a
+// column whose canonical distance ties with or beats a known P has
+//   L(b) <= P (1 + 2^-20 + 2 g) - |q|^2 (1 - a/2 - (d/32 + 8) 2^-23) + 2^-100
+// (the last factor covers |q|^2's own rounding, 2^-100 every underflow).  k_certify evaluates
+// every column that meets this; samples with too many of them, or out of the
+// bound's range, go to k_scan_exact's list form.
+
+// samples per launch of the certified scan: bounds its scratch (about 100 MB of
+// candidates) whatever |A| is; 128 sample tiles still fill the SMs
+constexpr int64_t kCertSlice = 16384;
+
+bool exact_tc_supported(const ch_set* A, const ch_set* B, int64_t T) {
+  if (A->dtype != B->dtype || (A->dtype != CH_F32 && A->dtype != CH_BF16)) return false;
+  const int64_t row = int64_t(A->d) * int64_t(elem_size(A->dtype));
+  if (A->d <= 4 || row % 16 != 0 || row > 16384) return false;
+  if ((reinterpret_cast<uintptr_t>(A->data) & 15) || (reinterpret_cast<uintptr_t>(B->data) & 15)) return false;
+  return T >= 1 && B->n >= kBN && B->n < (int64_t(1) << 31) && T * B->n >= (int64_t(1) << 20);
+}
+
+static int cert_screen(int dtype) { return dtype == CH_F32 ? CH_SCREEN_TF32 : CH_SCREEN_BF16; }
+
+size_t exact_tc_workspace(int64_t T, int64_t nB, int d, int dtype, int sm_count, int chunk_sms) {
+  const int64_t Ts = std::min(T, kCertSlice);
+  // the slices' plans differ in their tile count: room for the most chunks
+  size_t parts = 0;
+  for (int64_t t : {Ts, T % kCertSlice ? T % kCertSlice : Ts}) {
+    const Plan p = make_plan(t, nB, d, 1, sm_count, chunk_sms, cert_screen(dtype));
+    parts = std::max(parts, size_t(kSlices * p.chunks) * t * kClasses);
+  }
+  return ((size_t(Ts) * d * elem_size(dtype) + 255) & ~size_t(255)) + 3 * ((parts * 4 + 255) & ~size_t(255)) +
+         ((size_t(T) * 4 + 255) & ~size_t(255)) + ((size_t(T) * 8 + 255) & ~size_t(255)) + 1024;
+}
+
+void launch_exact_tc(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const float* normB, void* work,
+                     float* min_d, int64_t* argmin, int sm_count, int chunk_sms, cudaStream_t s, long long wait_cycles) {
+  if (T == 0) return;
+  const int screen = cert_screen(A->dtype);
+  const int es = static_cast<int>(elem_size(A->dtype)), d = A->d, row_bytes = d * es;
+  const int64_t Ts = std::min(T, kCertSlice);
+  auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
+  char* w = static_cast<char*>(work);
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(w);  // [0] listed samples, [1] a screen gave up
+  w += 256;
+  int32_t* list = reinterpret_cast<int32_t*>(w);
+  w += al(size_t(T) * 4);
+  unsigned long long* best = reinterpret_cast<unsigned long long*>(w);
+  w += al(size_t(T) * 8);
+  uint8_t* Q = reinterpret_cast<uint8_t*>(w);
+  w += al(size_t(Ts) * row_bytes);
+  CHX_CUDA(cudaMemsetAsync(ctl, 0, 8, s));
+
+  const double c_in = screen == CH_SCREEN_TF32 ? 0x1p-9 * (1.0 + 0x1p-10) : 0.0;
+  const double a_half = (c_in + 4.0 * d * 0x1p-23) + 0x1p-23;
+  CertArgs c;
+  c.d = d;
+  c.nB = B->n;
+  c.p_scale = 1.0 + 0x1p-20 + 2.0 * (ceil_div(d, 32) + 9) * 0x1p-24;
+  c.q_scale = 1.0 - a_half - (ceil_div(d, 32) + 8) * 0x1p-23;
+  c.list = list;
+  c.ctl = ctl;
+  c.best = best;
+  c.limit = std::min<int64_t>(2048, std::max<int64_t>(256, B->n / 8));
+  for (int64_t l0 = 0; l0 < T; l0 += kCertSlice) {
+    const int64_t n = std::min(kCertSlice, T - l0);
+    const Plan p = make_plan(n, B->n, d, 1, sm_count, chunk_sms, screen);
+    const size_t parts = size_t(kSlices * p.chunks) * n * kClasses;
+    char* v = w;
+    ScreenArgs a;
+    a.part_s = reinterpret_cast<float*>(v);
+    v += al(parts * 4);
+    a.part_i = reinterpret_cast<int32_t*>(v);
+    v += al(parts * 4);
+    a.part_2 = reinterpret_cast<float*>(v);
+    const void* q = Q;
+    if (qidx) {
+      const int64_t words = n * (row_bytes / 16);
+      launch_k(k_gather_rows, static_cast<int>(ceil_div(words, 256)), 256, 0, s, static_cast<const uint8_t*>(A->data),
+               A->scales, A->n, row_bytes, qidx + l0, n, Q, static_cast<float*>(nullptr));
+      launch_check("gather_rows");
+    } else {  // the samples are A's rows in order
+      q = static_cast<const uint8_t*>(A->data) + size_t(l0) * row_bytes;
+    }
+    const CUtensorMap tmQ = make_map(q, A->dtype, n, d, kBM);
+    const CUtensorMap tmB = make_map(B->data, B->dtype, B->n, d, kBN);
+    a.T = n;
+    a.nB = B->n;
+    a.kblocks = p.kblocks;
+    a.last_steps = last_steps_of(row_bytes);
+    a.row_tiles = p.row_tiles;
+    a.chunks = p.chunks;
+    a.chunk_len = p.chunk_len;
+    a.stages = p.stages;
+    a.stream_q = p.stream_q ? 1 : 0;
+    a.normB = normB;
+    a.scaleB = nullptr;
+    a.scaleQ = nullptr;
+    a.shrink = static_cast<float>((1.0 - a_half - (d + 2) * 0x1p-23) * (1.0 - 0x1p-23));
+    a.status = ctl + 1;
+    a.fail_bit = 1u;
+    a.wait_cycles = wait_cycles > 0 ? wait_cycles : kTimeoutCycles;
+    auto run = [&](auto kern) {
+      CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)); /* constant */
+      launch_k(kern, p.grid, kThreads, p.smem, s, tmQ, tmB, a);
+    };
+    if (screen == CH_SCREEN_TF32)
+      p.stream_q ? run(k_screen<CH_SCREEN_TF32, true, true>) : run(k_screen<CH_SCREEN_TF32, false, true>);
+    else
+      p.stream_q ? run(k_screen<CH_SCREEN_BF16, true, true>) : run(k_screen<CH_SCREEN_BF16, false, true>);
+    launch_check("screen");
+    c.l0 = l0;
+    c.T = n;
+    c.part_s = a.part_s;
+    c.part_i = a.part_i;
+    c.part_2 = a.part_2;
+    c.parts = kSlices * p.chunks;
+    c.slices = kSlices;
+    c.chunk_len = p.chunk_len;
+    c.tile = kBN;
+    launch_certify(A, qidx, B, c, min_d, argmin, s);
+  }
+  launch_scan_list(A, qidx, T, B, list, ctl, best, min_d, argmin, sm_count, s);
 }
 
 }  // namespace chx

@@ -33,7 +33,7 @@
 #include "common.cuh"
 
 namespace chx {
-size_t estimate_footprint(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p);
+size_t estimate_footprint(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p, bool plain);
 }
 
 using Clock = std::chrono::steady_clock;
@@ -126,12 +126,19 @@ ch_status run_request(ch_server* s, ch_ctx* c, Request& r, double* eta) {
   if (s->fault == Fault::slow) std::this_thread::sleep_for(std::chrono::milliseconds(50));
   void* ws = nullptr;
   if (cudaSetDevice(c->device) != cudaSuccess) return CH_ECUDA;
-  if (cudaMallocFromPoolAsync(&ws, r.footprint + 256, s->main->pool, c->stream) != cudaSuccess) {
+  size_t bytes = r.footprint;
+  cudaError_t got = cudaMallocFromPoolAsync(&ws, bytes + 256, s->main->pool, c->stream);
+  if (got != cudaSuccess) {  // once more with the exact scan's CUDA-core form
+    cudaGetLastError();
+    bytes = std::min(bytes, chx::estimate_footprint(c, A, B, &r.p, true));
+    got = cudaMallocFromPoolAsync(&ws, bytes + 256, s->main->pool, c->stream);
+  }
+  if (got != cudaSuccess) {
     cudaGetLastError();
     return CH_ENOMEM;
   }
   c->ws.base = static_cast<char*>(ws);
-  c->ws.cap = r.footprint + 256;
+  c->ws.cap = bytes + 256;
   c->ws.used = 0;
   c->ws.borrowed = true;
   const ch_status st = ch_estimate(c, A, B, &r.p, eta, nullptr);
@@ -261,7 +268,10 @@ ch_status ch_serve_submit(ch_server* s, uint64_t setA, uint64_t setB, const ch_e
     const ch_set* B = ib->second;
     if (A->d != B->d || A->dtype != B->dtype || B->n < 1) return CH_EINVAL;
     if (p->T < 0 || (p->T == 0 && !(p->eps > 0.0 && p->eps < 1.0))) return CH_EINVAL;
-    r->footprint = chx::estimate_footprint(s->slot_ctx[0], A, B, p);
+    r->footprint = chx::estimate_footprint(s->slot_ctx[0], A, B, p, false);
+    // a budget too small for the exact scan's tensor-core form gets its CUDA-core form
+    if (int64_t(r->footprint) > s->cfg.hbm_budget_bytes)
+      r->footprint = chx::estimate_footprint(s->slot_ctx[0], A, B, p, true);
     if (s->fault == Fault::admit || int64_t(r->footprint) > s->cfg.hbm_budget_bytes) {
       ++s->rejected;
       return CH_EBUSY;
