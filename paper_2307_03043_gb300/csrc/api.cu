@@ -502,17 +502,25 @@ static void take_scan(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, int64
   sb->cert = sb->screen == CH_SCREEN_EXACT && metric == CH_L2 && !plain && !c->exact_plain &&
              exact_tc_supported(A, B, T);
   if (sb->cert) {
-    sb->part = ScanPart{nullptr, nullptr, 0};
+    sb->part = ScanPart{nullptr, nullptr, 0, nullptr};
     sb->screen_work =
         lay.template take<char>(exact_tc_workspace(T, B->n, A->d, A->dtype, c->sm_count, c->screen_chunk_sms));
     sb->norms = norms_usable(c, B) ? nullptr : lay.template take<float>(size_t(B->n));
   } else if (sb->screen == CH_SCREEN_EXACT) {
     sb->part.chunks = scan_exact_chunks(T, B->n, A->d, A->dtype, c->sm_count);
-    sb->part.val = lay.template take<float>(size_t(sb->part.chunks) * std::max<int64_t>(T, 1));
-    sb->part.idx = lay.template take<int64_t>(size_t(sb->part.chunks) * std::max<int64_t>(T, 1));
+    sb->part.val = nullptr;
+    sb->part.idx = nullptr;
+    sb->part.best = nullptr;
+    if (A->d <= kScanSmallMaxD) {
+      sb->part.best =
+          lay.template take<unsigned long long>(size_t(scan_small_segments(B->n)) * std::max<int64_t>(T, 1));
+    } else {
+      sb->part.val = lay.template take<float>(size_t(sb->part.chunks) * std::max<int64_t>(T, 1));
+      sb->part.idx = lay.template take<int64_t>(size_t(sb->part.chunks) * std::max<int64_t>(T, 1));
+    }
     sb->screen_work = nullptr;
   } else {
-    sb->part = ScanPart{nullptr, nullptr, 0};
+    sb->part = ScanPart{nullptr, nullptr, 0, nullptr};
     sb->screen_work =
         lay.template take<char>(screen_workspace(T, B->n, A->d, static_cast<int>(R), c->sm_count,
                                                  c->screen_chunk_sms, sb->screen));
@@ -534,7 +542,7 @@ static void run_scan(ch_ctx* c, const ch_set* A, const int64_t* idx, int64_t T, 
     timer.start(c->stream);
     launch_scan_exact(A, idx, T, B, metric, sb->part, c->sm_count, c->stream);
     timer.stop(c->stream);
-    launch_scan_merge(sb->part, T, idx, m, argmin, c->stream);
+    launch_scan_merge(sb->part, T, B->n, idx, m, argmin, c->stream);
   } else {
     ensure_norms(const_cast<ch_set*>(B), c->stream);
     launch_screen_l2(A, idx, T, B, sb->screen, static_cast<int>(R), sb->screen_work, m, argmin, status, c->sm_count,
@@ -1229,7 +1237,7 @@ static void run_small_scans(ch_ctx* c, const std::vector<int64_t>& run, const st
   std::map<std::tuple<int, int, int>, std::vector<int64_t>> groups;
   for (int64_t i : run)
     if (small[i]) groups[{A[i]->dtype, params[i].hash.metric, A[i]->d}].push_back(i);
-  const int spi = small_scan_samples_per_item();
+  const int64_t most = small_scan_max_groups();
   for (auto& g : groups) {
     const auto& ids = g.second;
     const int dtype = std::get<0>(g.first), metric = std::get<1>(g.first), d = std::get<2>(g.first);
@@ -1246,10 +1254,20 @@ static void run_small_scans(ch_ctx* c, const std::vector<int64_t>& run, const st
       std::vector<SmallScanItem> it;
       for (size_t j = 0; j < ids.size(); ++j) {
         const int64_t i = ids[j];
-        const int64_t sb = ceil_div(Ts[i], int64_t(spi));
+        // the samples' groups of 256 in equal shares (2219 samples, 9 groups: 5 + 4, not 8 + 1)
+        const int64_t G = ceil_div(Ts[i], int64_t(256)), parts = ceil_div(G, most);
         for (int64_t b0 = 0; b0 < B[i]->n; b0 += cl)
-          for (int64_t q = 0; q < sb; ++q) it.push_back(SmallScanItem{int32_t(j), int32_t(q), b0});
+          for (int64_t q = 0; q < parts; ++q) {
+            const int64_t g0 = q * G / parts, g1 = (q + 1) * G / parts;
+            it.push_back(SmallScanItem{int32_t(j), int32_t(g0), int32_t(g1 - g0), 0, b0});
+          }
       }
+      // largest first, so that the blocks finish together
+      auto cost = [&](const SmallScanItem& e) {
+        return std::min(cl, B[ids[e.pair]]->n - e.b0) * (e.groups + 1);
+      };
+      std::stable_sort(it.begin(), it.end(),
+                       [&](const SmallScanItem& x, const SmallScanItem& y) { return cost(x) > cost(y); });
       return it;
     };
     // device buffers: the pair list and the largest item list of the candidates
@@ -1265,10 +1283,11 @@ static void run_small_scans(ch_ctx* c, const std::vector<int64_t>& run, const st
     }
     char* dmem = nullptr;
     const size_t pbytes = (sizeof(SmallScanPair) * pairs.size() + 255) & ~size_t(255);
-    CHX_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&dmem), pbytes + sizeof(SmallScanItem) * max_items,
-                                     c->pool, c->stream));
+    CHX_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&dmem),
+                                     pbytes + 256 + sizeof(SmallScanItem) * max_items, c->pool, c->stream));
     SmallScanPair* dp = reinterpret_cast<SmallScanPair*>(dmem);
-    SmallScanItem* di = reinterpret_cast<SmallScanItem*>(dmem + pbytes);
+    unsigned int* next = reinterpret_cast<unsigned int*>(dmem + pbytes);
+    SmallScanItem* di = reinterpret_cast<SmallScanItem*>(dmem + pbytes + 256);
     CHX_CUDA(cudaMemcpyAsync(dp, pairs.data(), sizeof(SmallScanPair) * pairs.size(), cudaMemcpyHostToDevice,
                              c->stream));
     float best_ms = 0.0f;
@@ -1277,8 +1296,8 @@ static void run_small_scans(ch_ctx* c, const std::vector<int64_t>& run, const st
       CHX_CUDA(cudaMemcpyAsync(di, lists[k].data(), sizeof(SmallScanItem) * lists[k].size(), cudaMemcpyHostToDevice,
                                c->stream));
       if (cands.size() > 1) CHX_CUDA(cudaEventRecord(c->ev[5], c->stream));
-      launch_scan_small_batch(dp, di, static_cast<int64_t>(lists[k].size()), cands[k], dtype, metric, d, c->sm_count,
-                              c->stream);
+      launch_scan_small_batch(dp, di, static_cast<int64_t>(lists[k].size()), cands[k], dtype, metric, d, next,
+                              c->sm_count, c->stream);
       if (cands.size() > 1) {
         CHX_CUDA(cudaEventRecord(c->ev[6], c->stream));
         CHX_CUDA(cudaEventSynchronize(c->ev[6]));

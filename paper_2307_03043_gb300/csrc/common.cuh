@@ -279,6 +279,13 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+// a + b, per half (a fused multiply-add by one, so that no multiplication before or
+// after it can be fused with it)
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(0x3F8000003F800000ull), "l"(b));
+  return r;
+}
 // min(a, b, c) in one instruction (sm_100 and later); like fminf, a NaN operand
 // is ignored when another is a number
 __device__ __forceinline__ float fmin3(float a, float b, float c) {
@@ -500,15 +507,20 @@ void launch_rerank(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set
                    const int32_t* part_i, int parts, int per, int occ, int stride, int R, float* min_d,
                    int64_t* argmin, cudaStream_t s);
 
-// exact scan: per (sample, chunk) minima, then merge
+// exact scan: per (sample, chunk) minima, then merge; the small-d scan (d <= 4)
+// folds every chunk's minimum into best [T] = (distance bits, index) instead
+constexpr int kScanSmallMaxD = 4;
 struct ScanPart {
   float* val;
   int64_t* idx;
   int chunks;
+  unsigned long long* best;
 };
 void launch_scan_exact(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, ScanPart part,
                        int sm_count, cudaStream_t s);
-void launch_scan_merge(ScanPart part, int64_t T, const int64_t* qidx, float* min_d, int64_t* argmin,
+// segments of 2^31 rows of B that the small-d scan keeps minima for (best holds T words each)
+int scan_small_segments(int64_t nB);
+void launch_scan_merge(ScanPart part, int64_t T, int64_t nB, const int64_t* qidx, float* min_d, int64_t* argmin,
                        cudaStream_t s);
 int scan_exact_chunks(int64_t T, int64_t nB, int d, int dtype, int sm_count);
 
@@ -523,19 +535,22 @@ struct SmallScanPair {
   const void* B;
   const float* scB;
   int64_t nB;
-  unsigned long long* best;  // [T] min over B of canonical distance bits << 32, preset to all ones
+  unsigned long long* best;  // [T] min over B of (canonical distance bits << 32 | index), preset to all ones
 };
 struct SmallScanItem {
   int32_t pair;    // index into the pair list
-  int32_t sblock;  // block of samples
+  int32_t group;   // first group of 256 samples
+  int32_t groups;  // groups of the item, 1 .. small_scan_max_groups()
+  int32_t pad;
   int64_t b0;      // first point of B of the item's chunk
 };
-// samples per item of the batched small scan
-int small_scan_samples_per_item();
+int small_scan_max_groups();
 // one persistent launch over every item (all pairs of one storage type, metric
-// and dimension d <= 4); each item's minimum distances fold into best[] by atomicMin
+// and dimension d <= 4); each item's minima fold into best[] by atomicMin; next: a
+// device word the items are counted out with
 void launch_scan_small_batch(const SmallScanPair* pairs, const SmallScanItem* items, int64_t n_items,
-                             int64_t chunk_len, int dtype, int metric, int d, int sm_count, cudaStream_t s);
+                             int64_t chunk_len, int dtype, int metric, int d, unsigned int* next, int sm_count,
+                             cudaStream_t s);
 
 // tensor-core screen + rerank (l2)
 bool screen_supported(int screen, const ch_set* A, const ch_set* B);

@@ -25,8 +25,8 @@ def ctx():
     ch.ch_ctx_destroy(c)
 
 
-def _scan(ctx, A, B, idx, dtype=ch.CH_F32):
-    """(min_d, argmin) of the exact l2 scan on the GPU, and the values the library saw."""
+def _scan(ctx, A, B, idx, dtype=ch.CH_F32, metric=ch.CH_L2):
+    """(min_d, argmin) of the exact scan on the GPU, and the values the library saw."""
     T = idx.size
     if dtype == ch.CH_BF16:
         hA, hB = workloads.to_bf16_bits(A), workloads.to_bf16_bits(B)
@@ -38,17 +38,17 @@ def _scan(ctx, A, B, idx, dtype=ch.CH_F32):
     sB = ch.ch_set_create(ctx, dB, 2, B.shape[0], B.shape[1], dtype)
     m = torch.full((T,), -1.0, device="cuda")
     am = torch.full((T,), -7, dtype=torch.int64, device="cuda")
-    ch.ch_sampled_nn(ctx, sA, torch.from_numpy(idx).cuda(), T, sB, ch.CH_L2, ch.CH_SCREEN_EXACT, 8, m, am)
+    ch.ch_sampled_nn(ctx, sA, torch.from_numpy(idx).cuda(), T, sB, metric, ch.CH_SCREEN_EXACT, 8, m, am)
     out = m.cpu().numpy(), am.cpu().numpy()
     ch.ch_set_destroy(sA)
     ch.ch_set_destroy(sB)
     return out, A, B
 
 
-def _check(ctx, A, B, idx, dtype=ch.CH_F32):
-    (m, am), A, B = _scan(ctx, A, B, idx, dtype)
+def _check(ctx, A, B, idx, dtype=ch.CH_F32, metric=ch.CH_L2):
+    (m, am), A, B = _scan(ctx, A, B, idx, dtype, metric)
     ok = idx >= 0
-    mo, amo = oracle.scan(A, idx[ok], B, ch.CH_L2)
+    mo, amo = oracle.scan(A, idx[ok], B, metric)
     assert np.array_equal(m[ok].view(np.uint32), mo.view(np.uint32))
     assert np.array_equal(am[ok], amo)
     assert np.all(m[~ok] == 0) and np.all(am[~ok] == -1)
@@ -92,6 +92,34 @@ def test_certified_scan_data(ctx, case):
         B[100:700] = A
     idx = np.random.default_rng(1).integers(0, 600, 1300).astype(np.int64)
     _check(ctx, A, B, idx)
+
+
+@pytest.mark.parametrize("metric", [ch.CH_L1, ch.CH_L2], ids=["l1", "l2"])
+@pytest.mark.parametrize("d", [1, 2, 3, 4])
+@pytest.mark.parametrize("case", ["plain", "duplicates", "offset", "offset_mixed", "tiny", "huge", "few_rows"])
+def test_small_d_scan_data(ctx, metric, d, case):
+    """d <= 4: sub-tile minima under the error bound, with the second-best sub-tile
+    and whole-chunk evaluations that ties, offsets and extreme magnitudes call for."""
+    A, B = workloads.gaussian_mixture(700, 5000, d, 21 + d, clusters=4)
+    if case == "duplicates":
+        B[2500:] = B[:2500]
+    elif case == "offset":
+        A += 3000
+        B += 3000
+    elif case == "offset_mixed":
+        A[::2] += 3000
+        B[::3] += 3000
+    elif case == "tiny":
+        A *= np.float32(1e-22)
+        B *= np.float32(1e-22)
+    elif case == "huge":
+        A = (A * 1e-3 + 2e19).astype(np.float32)
+        B = (B * 1e-3 + 2e19).astype(np.float32)
+    elif case == "few_rows":
+        B = B[:33]
+    idx = np.random.default_rng(4).integers(0, 700, 1500).astype(np.int64)
+    idx[2::37] = -1
+    _check(ctx, A, B, idx, metric=metric)
 
 
 def test_certified_brute_force_over_slices(ctx):
