@@ -311,19 +311,51 @@ void launch_draws(const uint64_t* prefix, int64_t nA, const uint64_t* W, int64_t
 // binary64 summation order is the same on every GPU:
 //   out[0] = (1/T) sum_l m_l W / w_{x_l};  out[1] = sum_a D_a.
 // Block b sums the contiguous slices [b*len, (b+1)*len) of the samples and of D.
-__device__ inline void block_sum2(double& a, double& b, double* sa, double* sb) {
-  sa[threadIdx.x] = a;
-  sb[threadIdx.x] = b;
-  __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-    if (threadIdx.x < st) {
-      sa[threadIdx.x] += sa[threadIdx.x + st];
-      sb[threadIdx.x] += sb[threadIdx.x + st];
-    }
-    __syncthreads();
+// One summation order everywhere: 256 values v[t] by the halving tree
+// v[t] += v[t + st], st = 128 .. 1.  The helpers below run it on one warp, lane t
+// holding v[t + 32 k], k < 8, in registers: the steps 128, 64 and 32 pair registers
+// and the others lanes.  n: values from index n on are exactly zero, so the steps
+// that would only add zeros to the first n are left out (x + 0 = x for the sums
+// here, which are never -0); FP64 adds are slow enough on this GPU for that to pay.
+__device__ __forceinline__ double warp_tree(double (&v)[8], int64_t n) {
+  if (n > 128) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += v[k + 4];
   }
-  a = sa[0];
-  b = sb[0];
+  if (n > 64) {
+    v[0] += v[2];
+    v[1] += v[3];
+  }
+  if (n > 32) v[0] += v[1];
+#pragma unroll
+  for (int st = 16; st > 0; st >>= 1) v[0] += __shfl_down_sync(0xFFFFFFFFu, v[0], st);
+  return v[0];  // the sum, on lane 0
+}
+
+// the tree over one value pair per thread of a 256-thread block (n as above): one
+// barrier, then the tree on warps 0 (a) and 1 (b); lane 0 of each returns its sum
+__device__ __forceinline__ double block_tree2(double a, double b, int64_t na, int64_t nb, double* s_a, double* s_b) {
+  s_a[threadIdx.x] = a;
+  s_b[threadIdx.x] = b;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x < 64) {
+    const double* src = threadIdx.x < 32 ? s_a : s_b;
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = src[(threadIdx.x & 31) + 32 * k];
+    r = warp_tree(v, threadIdx.x < 32 ? na : nb);
+  }
+  return r;
+}
+
+// the tree over the kCombineBlocks partials out[2 + 2 b + which], by one warp
+__device__ __forceinline__ double partial_tree(const double* out, int which) {
+  static_assert(kCombineBlocks == 128, "four partials per lane");
+  double v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = k < 4 ? __ldcg(&out[2 + 2 * ((threadIdx.x & 31) + 32 * k) + which]) : 0.0;
+  return warp_tree(v, kCombineBlocks);
 }
 
 // the result block from the summed partials (thread 0)
@@ -348,14 +380,12 @@ __device__ inline void combine_write(double a, double b, const uint64_t* Wp, int
 }
 
 // With ticket (a zeroed counter): the block that finishes last also sums the
-// kCombineBlocks partials, with the same tree as k_combine_final (256 threads,
-// the upper half adding exact zeros), so one launch does both passes.
+// kCombineBlocks partials, so one launch does both passes.
 __global__ void __launch_bounds__(256) k_combine_part(const float* m, const int64_t* idx, const uint64_t* w,
                                                       const uint64_t* Wp, int64_t T, const float* D, int64_t nA,
                                                       double* out, uint32_t* ticket, CollectArgs collect) {
   pdl_entry();
   __shared__ double s_a[256], s_b[256];
-  __shared__ bool s_last;
   const uint64_t W = Wp ? *Wp : 0;
   const int64_t lt = ceil_div_dev(T, kCombineBlocks), la = ceil_div_dev(nA, kCombineBlocks);
   double acc = 0.0, accD = 0.0;
@@ -369,35 +399,31 @@ __global__ void __launch_bounds__(256) k_combine_part(const float* m, const int6
     const int64_t end = min(nA, (blockIdx.x + 1) * la);
     for (int64_t a = blockIdx.x * la + threadIdx.x; a < end; a += blockDim.x) accD += static_cast<double>(D[a]);
   }
-  block_sum2(acc, accD, s_a, s_b);
-  if (threadIdx.x == 0) {
-    out[2 + 2 * blockIdx.x] = acc;
-    out[3 + 2 * blockIdx.x] = accD;
-  }
+  const double r = block_tree2(acc, accD, lt, la, s_a, s_b);
+  if (threadIdx.x >= 64) return;
+  const int which = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) out[2 + 2 * blockIdx.x + which] = r;
   if (!ticket) return;
+  __shared__ bool s_last;
   __threadfence();
-  __syncthreads();
+  asm volatile("bar.sync 1, 64;" ::: "memory");  // both partials are written
   if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == kCombineBlocks - 1;
-  __syncthreads();
+  asm volatile("bar.sync 1, 64;" ::: "memory");
   if (!s_last) return;
   __threadfence();
-  double a = 0.0, b = 0.0;
-  if (threadIdx.x < kCombineBlocks) {
-    a = __ldcg(&out[2 + 2 * threadIdx.x]);
-    b = __ldcg(&out[3 + 2 * threadIdx.x]);
-  }
-  __syncthreads();  // s_a / s_b are reused
-  block_sum2(a, b, s_a, s_b);
-  if (threadIdx.x == 0) combine_write(a, b, Wp, T, out, collect);
+  const double sum = partial_tree(out, which);
+  if (threadIdx.x == 32) s_b[0] = sum;
+  asm volatile("bar.sync 1, 64;" ::: "memory");
+  if (threadIdx.x == 0) combine_write(sum, s_b[0], Wp, T, out, collect);
 }
 
-__global__ void __launch_bounds__(kCombineBlocks) k_combine_final(const uint64_t* Wp, int64_t T, double* out,
-                                                                  CollectArgs c) {
+__global__ void __launch_bounds__(64) k_combine_final(const uint64_t* Wp, int64_t T, double* out, CollectArgs c) {
   pdl_entry();
-  __shared__ double s_a[kCombineBlocks], s_b[kCombineBlocks];
-  double a = out[2 + 2 * threadIdx.x], b = out[3 + 2 * threadIdx.x];
-  block_sum2(a, b, s_a, s_b);
-  if (threadIdx.x == 0) combine_write(a, b, Wp, T, out, c);
+  __shared__ double s_b;
+  const double sum = partial_tree(out, threadIdx.x >> 5);
+  if (threadIdx.x == 32) s_b = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) combine_write(sum, s_b, Wp, T, out, c);
 }
 
 void launch_combine(const float* m, const int64_t* idx, const uint64_t* w, const uint64_t* W, int64_t T,
@@ -410,7 +436,7 @@ void launch_combine(const float* m, const int64_t* idx, const uint64_t* w, const
   launch_k(k_combine_part, kCombineBlocks, 256, 0, s, m, idx, w, W, T, D, nA, out, static_cast<uint32_t*>(nullptr),
            collect);
   launch_check("combine_part");
-  launch_k(k_combine_final, 1, kCombineBlocks, 0, s, W, T, out, collect);
+  launch_k(k_combine_final, 1, 64, 0, s, W, T, out, collect);
   launch_check("combine_final");
 }
 
@@ -516,50 +542,63 @@ __global__ void __launch_bounds__(kBatchThreads) k_batch_sample(const BatchItem*
   }
 }
 
-// Per pair, 256 threads: the kCombineBlocks partial sums of k_combine_part (block
-// b's thread t sums the strided elements of slice b, then the block's tree), and
-// their final tree with the upper half of the threads adding zeros: the same
-// binary64 operations in the same order, so the same bits.
-__global__ void __launch_bounds__(256) k_batch_combine(const BatchItem* items) {
+// Per pair: the kCombineBlocks partial sums of k_combine_part, a warp per slice (its
+// lane t takes the threads t + 32 k of that slice's block), and their final tree:
+// the same binary64 operations in the same order, so the same bits.  Without block
+// barriers the slices' loads and divisions overlap (512 pairs of d = 3, 9.4k points:
+// 516 us with a block per slice in turn; see launch_batch_combine).
+constexpr int kBatchCombineThreads = 512;
+__global__ void __launch_bounds__(kBatchCombineThreads) k_batch_combine(const BatchItem* items) {
   pdl_entry();
-  __shared__ double s_a[256], s_b[256];
-  __shared__ double p_a[kCombineBlocks], p_b[kCombineBlocks];
+  __shared__ double part[2 + 2 * kCombineBlocks];  // laid out as k_combine_part's out
   const BatchItem it = items[blockIdx.x];
   const uint64_t W = it.res->W;
   const int64_t T = it.T, nA = it.nA;
   const int64_t lt = ceil_div_dev(T, kCombineBlocks), la = ceil_div_dev(nA, kCombineBlocks);
   const double Wd = static_cast<double>(W);
-  for (int b = 0; b < kCombineBlocks; ++b) {
-    double acc = 0.0, accD = 0.0;
+  const int lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; b < kCombineBlocks; b += kBatchCombineThreads / 32) {
+    double acc[8], accD[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] = accD[k] = 0.0;
     if (W != 0) {
       const int64_t end = min(T, (b + 1) * lt);
-      for (int64_t l = b * lt + threadIdx.x; l < end; l += blockDim.x) {
-        const float ml = it.mpk ? __uint_as_float(static_cast<uint32_t>(it.mpk[l] >> 32)) : it.m[l];
-        acc += static_cast<double>(ml) * (Wd / static_cast<double>(it.w[it.idx[l]]));
+      for (int64_t l0 = b * lt + lane; l0 < end; l0 += 256) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int64_t l = l0 + 32 * k;
+          if (l < end) {
+            const float ml = it.mpk ? __uint_as_float(static_cast<uint32_t>(it.mpk[l] >> 32)) : it.m[l];
+            acc[k] += static_cast<double>(ml) * (Wd / static_cast<double>(it.w[it.idx[l]]));
+          }
+        }
       }
     }
     const int64_t endA = min(nA, (b + 1) * la);
-    for (int64_t a = b * la + threadIdx.x; a < endA; a += blockDim.x) accD += static_cast<double>(it.D[a]);
-    block_sum2(acc, accD, s_a, s_b);
-    if (threadIdx.x == 0) {
-      p_a[b] = acc;
-      p_b[b] = accD;
+    for (int64_t a0 = b * la + lane; a0 < endA; a0 += 256) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (a0 + 32 * k < endA) accD[k] += static_cast<double>(it.D[a0 + 32 * k]);
     }
-    __syncthreads();  // s_a / s_b are reused
-  }
-  double a = 0.0, bsum = 0.0;
-  if (threadIdx.x < kCombineBlocks) {
-    a = p_a[threadIdx.x];
-    bsum = p_b[threadIdx.x];
+    const double sa = warp_tree(acc, lt), sd = warp_tree(accD, la);
+    if (lane == 0) {
+      part[2 + 2 * b] = sa;
+      part[3 + 2 * b] = sd;
+    }
   }
   __syncthreads();
-  block_sum2(a, bsum, s_a, s_b);
+  if (threadIdx.x >= 64) return;
+  double v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = k < 4 ? part[2 + 2 * (lane + 32 * k) + (threadIdx.x >> 5)] : 0.0;
+  const double sum = warp_tree(v, kCombineBlocks);
+  ResBlock* r = it.res;
   if (threadIdx.x == 0) {
-    ResBlock* r = it.res;
-    r->eta = (W != 0 && T > 0) ? a / static_cast<double>(T) : 0.0;
-    r->D_total = bsum;
+    r->eta = (W != 0 && T > 0) ? sum / static_cast<double>(T) : 0.0;
     if (it.statusA) r->statusA = *it.statusA;
     if (it.statusB) r->statusB = *it.statusB;
+  } else if (threadIdx.x == 32) {
+    r->D_total = sum;
   }
 }
 
@@ -571,7 +610,7 @@ void launch_batch_sample(const BatchItem* items, int64_t count, cudaStream_t s) 
 
 void launch_batch_combine(const BatchItem* items, int64_t count, cudaStream_t s) {
   if (count == 0) return;
-  launch_k(k_batch_combine, static_cast<int>(count), 256, 0, s, items);
+  launch_k(k_batch_combine, static_cast<int>(count), kBatchCombineThreads, 0, s, items);
   launch_check("batch_combine");
 }
 
