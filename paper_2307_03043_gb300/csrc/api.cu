@@ -1604,15 +1604,19 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
       CHX_CUDA(cudaStreamWaitEvent(c->stream, c->lanes[k]->ev[7], 0));
     }
   };
-  // one host thread per lane enqueues that lane's pairs (kernel launches are the
-  // host-side cost of small pairs); the sets' lazy state is already final
-  auto on_lanes = [&](auto&& body) {
+  // one host thread per lane enqueues that lane's pairs among those wanted (kernel
+  // launches are the host-side cost of small pairs; eight threads cost 0.5 ms to
+  // start and join, so lanes without pairs get none); the sets' lazy state is final
+  auto on_lanes = [&](auto&& wanted, auto&& body) {
+    std::vector<char> busy(K, 0);
+    for (int64_t i : run)
+      if (st[i] == CH_OK && wanted(i)) busy[i % K] = 1;
     std::vector<std::thread> th;
     for (int k = 0; k < K; ++k)
-      th.emplace_back([&, k] {
+      if (busy[k]) th.emplace_back([&, k] {
         cudaSetDevice(c->device);
         for (int64_t i : run) {
-          if (i % K != k || st[i] != CH_OK) continue;
+          if (i % K != k || st[i] != CH_OK || !wanted(i)) continue;
           try {
             body(c->lanes[k], i);
           } catch (const Err& e) {
@@ -1625,9 +1629,9 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
     for (auto& t : th) t.join();
   };
   fork();
-  on_lanes([&](ch_ctx* lane, int64_t i) {  // 1. CrudeNN (or the uniform baseline's equal weights)
+  // 1. CrudeNN (or the uniform baseline's equal weights); the batched launches follow below
+  on_lanes([&](int64_t i) { return !bcr[i]; }, [&](ch_ctx* lane, int64_t i) {
     const ch_est_params* p = &params[i];
-    if (bcr[i]) return;  // below, in the batched launches
     if (p->sampling == CH_SAMPLING_UNIFORM) {
       launch_fill_ones(Dp[i], A[i]->n, lane->stream);
       return;
@@ -1678,8 +1682,8 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
   }
   launch_batch_sample(ditems, static_cast<int64_t>(run.size()), c->stream);  // 2.
   fork();
-  on_lanes([&](ch_ctx* lane, int64_t i) {  // 3. the sampled scans (the small pairs' below)
-    if (small[i]) return;
+  // 3. the sampled scans (the small pairs' below)
+  on_lanes([&](int64_t i) { return !small[i]; }, [&](ch_ctx* lane, int64_t i) {
     const ch_est_params* p = &params[i];
     ScanBufs sc;
     carve(lane, [&](auto& lay) { take_scan(lay, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc); });
