@@ -322,7 +322,7 @@ static void take_crude(L& lay, const ch_set* A, const ch_set* B, const ch_hash_p
     cb->slots = nullptr;
     cb->keysA = lay.template take<uint64_t>(std::max<size_t>(size_t(nl) * A->n, 1));
     cb->keysB = lay.template take<uint64_t>(size_t(nl) * B->n);
-    cb->sort_work = lay.template take<char>(sort_window_workspace(A->n, B->n, nl));
+    cb->sort_work = lay.template take<char>(sort_group_workspace(B->n, nl));
     cb->cand = lay.template take<int32_t>(std::max<size_t>(size_t(A->n) * kw_k(hp) * kw_w(hp), 1));
     return;
   }
@@ -332,7 +332,7 @@ static void take_crude(L& lay, const ch_set* A, const ch_set* B, const ch_hash_p
     cb->slots = nullptr;
     cb->keysA = lay.template take<uint64_t>(std::max<size_t>(size_t(nl) * A->n, 1));
     cb->keysB = lay.template take<uint64_t>(size_t(nl) * B->n);
-    cb->sort_work = lay.template take<char>(sort_group_workspace(A->n, B->n, nl));
+    cb->sort_work = lay.template take<char>(sort_group_workspace(B->n, nl));
     return;
   }
   cb->plan = table_plan(B->n, nl);

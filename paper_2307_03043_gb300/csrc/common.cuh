@@ -379,14 +379,14 @@ void launch_keys_write(HashSrc X, int L, ScaleTables t, uint64_t* keys, cudaStre
 void launch_simhash_keys(const float* Y, int64_t n, int K, int L, uint64_t seed, uint64_t* keys, cudaStream_t s);
 
 // radix-sort grouping (CH_GROUP_SORT): keys [L][nA] and [L][nB] -> bidx, level
-size_t sort_group_workspace(int64_t nA, int64_t nB, int L);
+// (sort_group_workspace: scratch bytes, also of the k x W window below)
+size_t sort_group_workspace(int64_t nB, int L);
 bool sort_group_supported(int64_t nA, int64_t nB, int L);
 
 // k x W CrudeNN (Section 3): structure r's window of W points per a, by the same
 // sort, into cand[a * stride + r * W + q] (-1 past the retrieved points); level[a]
 // = the finest scale any structure so far found a point at (set by r = 0)
 constexpr int kWindowMax = 64;
-size_t sort_window_workspace(int64_t nA, int64_t nB, int L);
 void launch_sort_window(const uint64_t* keysA, int64_t nA, const uint64_t* keysB, int64_t nB, int L, int W, int r,
                         void* work, int32_t* cand, int stride, uint8_t* level, cudaStream_t s);
 // D_a = min over a's candidates of the canonical distance, b(a) its argmin

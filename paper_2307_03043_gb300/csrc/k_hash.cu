@@ -1501,8 +1501,11 @@ void launch_crude_dist(const ch_set* A, const ch_set* B, int metric, const int64
 // ------------------------------------------------------------------ k x W candidates
 // One warp per a: the canonical distance to each candidate (lane r sums
 // coordinates j = r mod 32, then the halving tree by shuffles), the minimum with
-// the smallest index on ties; one atomic per warp folds max D into *maxD.
-template <int DTA, int DTB, int METRIC>
+// the smallest index on ties; one atomic per warp folds max D into *maxD.  Lanes
+// read up to 32 candidates at once and drop empty places and repetitions (the k
+// structures find many of the same points); four of the rest at a time keep four
+// rows in flight.
+template <int DT, int METRIC>
 __global__ void __launch_bounds__(256) k_cand_dist(const void* A, const float* scA, int64_t nA, const void* B,
                                                    const float* scB, int d, const int32_t* cand, int stride,
                                                    int64_t* bidx, float* D, uint32_t* maxD) {
@@ -1512,20 +1515,42 @@ __global__ void __launch_bounds__(256) k_cand_dist(const void* A, const float* s
   if (a >= nA) return;
   float best = __int_as_float(0x7F800000);
   int64_t arg = INT64_MAX;
-  for (int c = 0; c < stride; ++c) {
-    const int32_t b = cand[a * stride + c];
-    if (b < 0) continue;
-    float p = 0.0f;
-    for (int j = lane; j < d; j += 32) {
-      const float t = __fsub_rn(load_elem<DTA>(A, a, d, j, scA), load_elem<DTB>(B, b, d, j, scB));
-      p = (METRIC == CH_L1) ? __fadd_rn(p, fabsf(t)) : __fmaf_rn(t, t, p);
-    }
+  for (int c0 = 0; c0 < stride; c0 += 32) {
+    const int32_t mine = c0 + lane < stride ? cand[a * stride + c0 + lane] : -1;
+    const unsigned same = __match_any_sync(0xFFFFFFFFu, mine);
+    unsigned left = __ballot_sync(0xFFFFFFFFu, mine >= 0 && lane == __ffs(same) - 1);
+    while (left) {
+      int64_t b[4];
+      bool live[4];
 #pragma unroll
-    for (int sh = 16; sh >= 1; sh >>= 1) p = __fadd_rn(p, __shfl_down_sync(0xFFFFFFFFu, p, sh));
-    const float v = __shfl_sync(0xFFFFFFFFu, (METRIC == CH_L1) ? p : __fsqrt_rn(p), 0);
-    if (v < best || (v == best && b < arg)) {
-      best = v;
-      arg = b;
+      for (int o = 0; o < 4; ++o) {
+        live[o] = left != 0;
+        b[o] = __shfl_sync(0xFFFFFFFFu, mine, live[o] ? __ffs(left) - 1 : 0);
+        if (!live[o]) b[o] = b[0];
+        left &= left - 1;
+      }
+      float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+      for (int j = lane; j < d; j += 32) {
+        const float x = load_elem<DT>(A, a, d, j, scA);
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const float t = __fsub_rn(x, load_elem<DT>(B, b[o], d, j, scB));
+          p[o] = (METRIC == CH_L1) ? __fadd_rn(p[o], fabsf(t)) : __fmaf_rn(t, t, p[o]);
+        }
+      }
+#pragma unroll
+      for (int sh = 16; sh >= 1; sh >>= 1)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) p[o] = __fadd_rn(p[o], __shfl_down_sync(0xFFFFFFFFu, p[o], sh));
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        const float v = __shfl_sync(0xFFFFFFFFu, (METRIC == CH_L1) ? p[o] : __fsqrt_rn(p[o]), 0);
+        if (live[o] && (v < best || (v == best && b[o] < arg))) {
+          best = v;
+          arg = b[o];
+        }
+      }
     }
   }
   if (lane == 0) {
@@ -1540,23 +1565,17 @@ void launch_cand_dist(const ch_set* A, const ch_set* B, int metric, const int32_
   if (maxD) CHX_CUDA(cudaMemsetAsync(maxD, 0, sizeof(uint32_t), s));
   if (A->n == 0) return;
   const int grid = static_cast<int>(ceil_div(A->n * 32, 256));
-  auto go = [&](auto dta, auto dtb) {
-    constexpr int DTA = decltype(dta)::value, DTB = decltype(dtb)::value;
-    if (metric == CH_L1)
-      launch_k(k_cand_dist<DTA, DTB, CH_L1>, grid, 256, 0, s, A->data, A->scales, A->n, B->data, B->scales, A->d, cand,
-                                                          stride, bidx, D, maxD);
-    else
-      launch_k(k_cand_dist<DTA, DTB, CH_L2>, grid, 256, 0, s, A->data, A->scales, A->n, B->data, B->scales, A->d, cand,
-                                                          stride, bidx, D, maxD);
+  auto go = [&](auto dt) {  // both sets have one storage type (checked by the caller)
+    constexpr int DT = decltype(dt)::value;
+    auto run = [&](auto kern) {
+      launch_k(kern, grid, 256, 0, s, A->data, A->scales, A->n, B->data, B->scales, A->d, cand, stride, bidx, D, maxD);
+    };
+    metric == CH_L1 ? run(k_cand_dist<DT, CH_L1>) : run(k_cand_dist<DT, CH_L2>);
   };
-  using F = std::integral_constant<int, CH_F32>;
-  using H = std::integral_constant<int, CH_BF16>;
-  using E = std::integral_constant<int, CH_FP8E4M3>;
-  // both sets have one storage type (checked by the caller)
   switch (A->dtype) {
-    case CH_F32: go(F{}, F{}); break;
-    case CH_BF16: go(H{}, H{}); break;
-    default: go(E{}, E{}); break;
+    case CH_F32: go(std::integral_constant<int, CH_F32>{}); break;
+    case CH_BF16: go(std::integral_constant<int, CH_BF16>{}); break;
+    default: go(std::integral_constant<int, CH_FP8E4M3>{}); break;
   }
   launch_check("cand_dist");
 }
