@@ -7,23 +7,165 @@ namespace chx {
 
 namespace {
 
-constexpr int kRerankWarps = 8;  // samples per block; each warp's candidate list in dynamic shared memory
+constexpr int kRerankWarps = 8;  // samples per block, a warp each
+
+// 16 bytes of a row as binary32 (FP8: times the row's scale)
+template <int DT>
+constexpr int kRowPer = DT == CH_F32 ? 4 : DT == CH_BF16 ? 8 : 16;
+template <int DT>
+__device__ __forceinline__ void row_vec(const void* row, int m, float sc, float (&v)[kRowPer<DT>]) {
+  const uint4 w = __ldg(static_cast<const uint4*>(row) + m);
+  const uint32_t q[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int e = 0; e < kRowPer<DT>; ++e) {
+    if constexpr (DT == CH_F32) v[e] = __uint_as_float(q[e]);
+    else if constexpr (DT == CH_BF16) v[e] = __uint_as_float(e & 1 ? q[e / 2] & 0xFFFF0000u : q[e / 2] << 16);
+    else v[e] = __fmul_rn(e4m3_to_f32(static_cast<uint8_t>(q[e / 4] >> (8 * (e % 4)))), sc);
+  }
+}
+
+// row a of a set, widened, into the warp's shared-memory row q [d]
+template <int DT>
+__device__ __forceinline__ void stage_query(float* q, const char* row, float sc, int d, int lane) {
+  for (int m = lane; m < d / kRowPer<DT>; m += 32) {
+    float v[kRowPer<DT>];
+    row_vec<DT>(row, m, sc, v);
+#pragma unroll
+    for (int e = 0; e < kRowPer<DT>; e += 4)
+      *reinterpret_cast<float4*>(q + m * kRowPer<DT> + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+  }
+  __syncwarp();
+}
+
+// Squared canonical l2 distances of the staged row q to up to 32 rows of B.  Two forms,
+// the same sums in the same order:
+//  * lane_dist, rows below 512 bytes: a row per lane, the 32 partials in its registers,
+//    no shuffles; a warp keeps 32 rows in flight.  Its loads touch a sector per lane, so
+//    wide rows outgrow L1 between them;
+//  * group_dist, wider rows: 32 / C lanes per row (C coordinates per 16-byte word), each
+//    owning C partials, so a row is read in whole 64- or 128-byte pieces; NR rows per
+//    lane group side by side.
+// Rerank of 8 entries x 4 columns for ~4.8k samples, cold caches, lane form / group form
+// / the earlier four rows per warp with a shuffle tree each: f32 d = 128 37 / 31 / 28 us
+// (the whole warm call 359 / 344 / 352 us), bf16 d = 384 122 / 67 / 65 us, bf16 d = 768
+// 256 / 97 / 94 us, fp8 d = 384 51 / - / 112 us.
+constexpr int kWideRow = 512;
+
+template <int DT>
+__device__ __forceinline__ float lane_dist(const float* __restrict__ q, const void* __restrict__ b, float sb, int d) {
+  constexpr int PER = kRowPer<DT>;
+  const int words = d / PER;
+  float p[32];
+#pragma unroll
+  for (int r = 0; r < 32; ++r) p[r] = 0.0f;
+#pragma unroll 1
+  for (int m0 = 0; m0 < words; m0 += 32 / PER) {
+#pragma unroll
+    for (int m = 0; m < 32 / PER; ++m)
+      if (m0 + m < words) {
+        float y[PER];
+        row_vec<DT>(b, m0 + m, sb, y);
+#pragma unroll
+        for (int e = 0; e < PER; e += 4) {
+          const float4 x = *reinterpret_cast<const float4*>(q + (m0 + m) * PER + e);
+          const float xx[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float t = __fsub_rn(xx[k], y[e + k]);
+            p[m * PER + e + k] = __fmaf_rn(t, t, p[m * PER + e + k]);
+          }
+        }
+      }
+  }
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1)
+#pragma unroll
+    for (int r = 0; r < s; ++r) p[r] = __fadd_rn(p[r], p[r + s]);
+  return p[0];
+}
+
+// cols [32] in shared memory (entries from ncols on are ignored): the distance of row
+// cols[lane] on every lane < ncols
+template <int DT>
+__device__ __forceinline__ float group_dist(const float* __restrict__ q, const char* __restrict__ B, size_t row_bytes,
+                                            const float* __restrict__ scB, const int32_t* cols, int ncols, int d) {
+  constexpr int C = kRowPer<DT>, LPR = 32 / C, G = 32 / LPR, NR = DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1;
+  const int lane = threadIdx.x & 31, sub = lane % LPR, grp = lane / LPR;
+  const int chunks = d / C;
+  float mine = 0.0f;
+  for (int base = 0; base < ncols; base += G * NR) {
+    const void* row[NR];
+    float sb[NR], p[NR][C];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      const int at = base + k * G + grp;
+      const int64_t b = cols[at < ncols ? at : 0];
+      row[k] = B + size_t(b) * row_bytes;
+      sb[k] = DT == CH_FP8E4M3 ? scB[b] : 1.0f;
+#pragma unroll
+      for (int i = 0; i < C; ++i) p[k][i] = 0.0f;
+    }
+#pragma unroll 4
+    for (int m = sub; m < chunks; m += LPR) {
+      float x[C];
+#pragma unroll
+      for (int e = 0; e < C; e += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(q + m * C + e);
+        x[e] = t.x;
+        x[e + 1] = t.y;
+        x[e + 2] = t.z;
+        x[e + 3] = t.w;
+      }
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        float y[C];
+        row_vec<DT>(row[k], m, sb[k], y);
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          const float t = __fsub_rn(x[i], y[i]);
+          p[k][i] = __fmaf_rn(t, t, p[k][i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+#pragma unroll
+      for (int s = 16; s >= C; s >>= 1)
+#pragma unroll
+        for (int i = 0; i < C; ++i) p[k][i] = __fadd_rn(p[k][i], __shfl_down_sync(0xFFFFFFFFu, p[k][i], s / C, LPR));
+#pragma unroll
+      for (int s = C / 2; s >= 1; s >>= 1)
+#pragma unroll
+        for (int i = 0; i < s; ++i) p[k][i] = __fadd_rn(p[k][i], p[k][i + s]);
+      // group g's sum sits on its first lane and belongs to column base + k G + g
+      const int g = lane - base - k * G;
+      const float v = __shfl_sync(0xFFFFFFFFu, p[k][0], (g >= 0 && g < G ? g : 0) * LPR);
+      if (g >= 0 && g < G) mine = v;
+    }
+  }
+  return mine;
+}
 
 // One warp per sample: the R best screened entries over all chunks (by s, then
 // index), the canonical binary32 distance of each of an entry's occ columns
-// (first column + o * stride, o < occ, columns < nB), and their minimum (ties:
-// smaller index).
-template <int DT, int METRIC>
+// (first column + o * stride, o < occ <= 4, columns < nB), and their minimum (ties:
+// smaller index).  Lane k holds the entries k, k + 32, ... and its smallest one; a
+// round takes the smallest of those by two integer minima and only the lane that
+// gave it looks its entries over again.  Eight entries then give every lane one column.
+template <int DT, bool WIDE>
 __global__ void __launch_bounds__(32 * kRerankWarps) k_rerank(const void* A, const float* scA, int64_t nA, const void* B,
                                                 const float* scB, int64_t nB, int d, const int64_t* idx, int64_t T,
                                                 const float* part_s, const int32_t* part_i, int parts, int per,
                                                 int occ, int stride, int R, float* min_d, int64_t* argmin) {
   pdl_entry();
-  extern __shared__ float s_dyn[];  // [kRerankWarps][parts * per] scores, then as many indices
+  extern __shared__ __align__(16) float s_dyn[];  // per warp: the query [d], scores and columns [parts * per]
+  __shared__ int32_t s_first[kRerankWarps][8], s_cols[WIDE ? kRerankWarps : 1][32];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nc = parts * per;
-  float* s_s = s_dyn + wib * nc;
-  int32_t* s_i = reinterpret_cast<int32_t*>(s_dyn + kRerankWarps * nc) + wib * nc;
+  float* q = s_dyn + size_t(wib) * ((d + 3) / 4 * 4 + 2 * nc);
+  uint32_t* s_s = reinterpret_cast<uint32_t*>(q + (d + 3) / 4 * 4);
+  int32_t* s_i = reinterpret_cast<int32_t*>(s_s + nc);
+  int32_t* first = s_first[wib];
   const int64_t l = int64_t(blockIdx.x) * kRerankWarps + wib;
   if (l >= T) return;
   const int64_t a = idx ? idx[l] : l;
@@ -34,81 +176,79 @@ __global__ void __launch_bounds__(32 * kRerankWarps) k_rerank(const void* A, con
     }
     return;
   }
+  const size_t row_bytes = size_t(d) * (DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1);
+  stage_query<DT>(q, static_cast<const char*>(A) + size_t(a) * row_bytes, DT == CH_FP8E4M3 ? scA[a] : 1.0f, d, lane);
+  // entries in integer order (-0 as +0; NaN scores and empty entries last), this lane's smallest
+  constexpr uint32_t kNone = 0xFFFFFFFFu;
+  uint32_t ms = kNone;
+  int32_t mi = INT32_MAX;
+  int mp = -1;
+  auto smaller = [&](uint32_t v, int32_t i, int p) {
+    if (v != kNone && (v < ms || (v == ms && i < mi))) {
+      ms = v;
+      mi = i;
+      mp = p;
+    }
+  };
+#pragma unroll 4
   for (int p = lane; p < nc; p += 32) {
     const int c = p / per, k = p % per;
     const size_t off = (size_t(c) * T + l) * per + k;
-    s_s[p] = part_s[off];
-    s_i[p] = part_i[off];
+    const float v = part_s[off];
+    const int32_t i = part_i[off];
+    const uint32_t e = i >= 0 && v == v ? ord_enc(v + 0.0f) : kNone;
+    s_s[p] = e;
+    s_i[p] = i;
+    smaller(e, i, p);
   }
-  __syncwarp();
-  float best = __int_as_float(0x7F800000);
-  int64_t bidx = INT64_MAX;
-  for (int round = 0; round < R; ++round) {
-    float ms = __int_as_float(0x7F800000);
-    int32_t mi = INT32_MAX;
-    int mp = -1;
-    for (int p = lane; p < nc; p += 32) {
-      const float v = s_s[p];
-      const int32_t i = s_i[p];
-      if (i >= 0 && (v < ms || (v == ms && i < mi))) {
-        ms = v;
-        mi = i;
-        mp = p;
+  float best = __int_as_float(0x7F800000);  // this lane's minimum and its column
+  uint32_t bcol = kNone;
+  for (int r0 = 0; r0 < R; r0 += 8) {
+    int n = 0;
+    for (; n < min(8, R - r0); ++n) {
+      const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, ms);
+      if (least == kNone) break;  // fewer than R entries
+      const int32_t col = __reduce_min_sync(0xFFFFFFFFu, ms == least ? mi : INT32_MAX);
+      if (lane == 0) first[n] = col;
+      if (ms == least && mi == col) {  // taken; columns are distinct, so one lane
+        s_s[mp] = kNone;
+        ms = kNone;
+        mi = INT32_MAX;
+        for (int p = lane; p < nc; p += 32) smaller(s_s[p], s_i[p], p);
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float os = __shfl_xor_sync(0xFFFFFFFFu, ms, o);
-      const int32_t oi = __shfl_xor_sync(0xFFFFFFFFu, mi, o);
-      const int op = __shfl_xor_sync(0xFFFFFFFFu, mp, o);
-      if (os < ms || (os == ms && oi < mi)) {
-        ms = os;
-        mi = oi;
-        mp = op;
-      }
-    }
-    if (mi == INT32_MAX || mi < 0) break;  // fewer than R entries
-    if (lane == (mp & 31)) s_i[mp] = -1;  // taken
     __syncwarp();
-    // canonical distances to the entry's columns, all at once (lane r sums
-    // coordinates j = r mod 32 of each; the reduction trees run side by side)
-    int64_t bo[kRerankMaxOcc];
-    bool vo[kRerankMaxOcc];
-    float part[kRerankMaxOcc];
-#pragma unroll
-    for (int o = 0; o < kRerankMaxOcc; ++o) {
-      bo[o] = int64_t(mi) + int64_t(o) * stride;
-      vo[o] = o < occ && bo[o] < nB;
-      part[o] = 0.0f;
+    int32_t col = -1;  // this lane's column
+    if ((lane >> 2) < n && (lane & 3) < occ) {
+      const int64_t b = int64_t(first[lane >> 2]) + int64_t(lane & 3) * stride;
+      if (b < nB) col = static_cast<int32_t>(b);
     }
-#pragma unroll 4
-    for (int j = lane; j < d; j += 32) {
-      const float x = load_elem<DT>(A, a, d, j, scA);
-#pragma unroll
-      for (int o = 0; o < kRerankMaxOcc; ++o) {
-        if (vo[o]) {
-          const float t = __fsub_rn(x, load_elem<DT>(B, bo[o], d, j, scB));
-          part[o] = (METRIC == CH_L1) ? __fadd_rn(part[o], fabsf(t)) : __fmaf_rn(t, t, part[o]);
-        }
+    float P = 0.0f;
+    if constexpr (WIDE) {
+      if (n > 0) {
+        int32_t* cols = s_cols[wib];
+        cols[lane] = col >= 0 ? col : first[0];
+        __syncwarp();
+        P = group_dist<DT>(q, static_cast<const char*>(B), row_bytes, scB, cols, 4 * n, d);
       }
+    } else if (col >= 0) {
+      P = lane_dist<DT>(q, static_cast<const char*>(B) + size_t(col) * row_bytes, DT == CH_FP8E4M3 ? scB[col] : 1.0f, d);
     }
-#pragma unroll
-    for (int sh = 16; sh >= 1; sh >>= 1) {
-#pragma unroll
-      for (int o = 0; o < kRerankMaxOcc; ++o) part[o] = __fadd_rn(part[o], __shfl_down_sync(0xFFFFFFFFu, part[o], sh));
-    }
-#pragma unroll
-    for (int o = 0; o < kRerankMaxOcc; ++o) {
-      const float dist = __shfl_sync(0xFFFFFFFFu, (METRIC == CH_L1) ? part[o] : __fsqrt_rn(part[o]), 0);
-      if (vo[o] && (dist < best || (dist == best && bo[o] < bidx))) {
+    if (col >= 0) {
+      const float dist = __fsqrt_rn(P);
+      if (dist < best || (dist == best && static_cast<uint32_t>(col) < bcol)) {
         best = dist;
-        bidx = bo[o];
+        bcol = static_cast<uint32_t>(col);
       }
     }
+    __syncwarp();
+    if (n < 8) break;
   }
+  const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(best));
+  bcol = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(best) == least ? bcol : kNone);
   if (lane == 0) {
-    min_d[l] = best;
-    if (argmin) argmin[l] = bidx;
+    min_d[l] = __uint_as_float(least);
+    if (argmin) argmin[l] = bcol == kNone ? INT64_MAX : static_cast<int64_t>(bcol);
   }
 }
 
@@ -119,73 +259,23 @@ void launch_rerank(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set
                    int64_t* argmin, cudaStream_t s) {
   CHX_CHECK(parts * per <= kRerankMaxCand && occ <= kRerankMaxOcc, CH_EINVAL, "rerank candidate list too long");
   const int blocks = static_cast<int>(ceil_div(T, kRerankWarps));
-  const size_t smem = size_t(kRerankWarps) * parts * per * 8;
-#define CHX_RERANK(DT)                                                                                        \
-  do {                                                                                                        \
-    CHX_CUDA(cudaFuncSetAttribute(k_rerank<DT, CH_L2>, cudaFuncAttributeMaxDynamicSharedMemorySize,             \
-                                  static_cast<int>(size_t(kRerankWarps) * kRerankMaxCand * 8)));               \
-    launch_k(k_rerank<DT, CH_L2>, blocks, 32 * kRerankWarps, smem, s, A->data, A->scales, A->n, B->data,        \
-             B->scales, B->n, A->d, qidx, T, part_s, part_i, parts, per, occ, stride, R, min_d, argmin);       \
-  } while (0)
-  if (A->dtype == CH_F32) CHX_RERANK(CH_F32);
-  else if (A->dtype == CH_BF16) CHX_RERANK(CH_BF16);
-  else CHX_RERANK(CH_FP8E4M3);
-#undef CHX_RERANK
+  const size_t smem = size_t(kRerankWarps) * ((size_t(A->d) + 3) / 4 * 4 + 2 * size_t(parts) * per) * 4;
+  auto run = [&](auto kern) {
+    // a constant value, so concurrent callers on other threads never race on it
+    CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(size_t(kRerankWarps) * (kMaxDim + 2 * kRerankMaxCand) * 4)));
+    launch_k(kern, blocks, 32 * kRerankWarps, smem, s, A->data, A->scales, A->n, B->data, B->scales, B->n, A->d, qidx, T,
+             part_s, part_i, parts, per, occ, stride, R, min_d, argmin);
+  };
+  const bool wide = size_t(A->d) * elem_size(A->dtype) >= kWideRow;
+  if (A->dtype == CH_F32) wide ? run(k_rerank<CH_F32, true>) : run(k_rerank<CH_F32, false>);
+  else if (A->dtype == CH_BF16) wide ? run(k_rerank<CH_BF16, true>) : run(k_rerank<CH_BF16, false>);
+  else wide ? run(k_rerank<CH_FP8E4M3, true>) : run(k_rerank<CH_FP8E4M3, false>);
   launch_check("rerank");
 }
 
 // ------------------------------------------------------------------ certified scan
 namespace {
-
-// 16 bytes of a row (4 binary32 or 8 bf16 coordinates) as binary32
-template <int DT>
-__device__ __forceinline__ void cert_vec(const void* row, int m, float (&v)[DT == CH_F32 ? 4 : 8]) {
-  const uint4 w = __ldg(static_cast<const uint4*>(row) + m);
-  if constexpr (DT == CH_F32) {
-    v[0] = __uint_as_float(w.x);
-    v[1] = __uint_as_float(w.y);
-    v[2] = __uint_as_float(w.z);
-    v[3] = __uint_as_float(w.w);
-  } else {
-    const uint32_t q[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      v[2 * e] = __uint_as_float(q[e] << 16);
-      v[2 * e + 1] = __uint_as_float(q[e] & 0xFFFF0000u);
-    }
-  }
-}
-
-// canonical squared l2 distance of two rows by one thread: the 32 partials in
-// registers, then the halving tree
-template <int DT>
-__device__ __forceinline__ float cert_dist(const void* q, const void* b, int d) {
-  constexpr int PER = DT == CH_F32 ? 4 : 8;
-  const int words = d / PER;
-  float p[32];
-#pragma unroll
-  for (int r = 0; r < 32; ++r) p[r] = 0.0f;
-#pragma unroll 1
-  for (int m0 = 0; m0 < words; m0 += 32 / PER) {
-#pragma unroll
-    for (int m = 0; m < 32 / PER; ++m)
-      if (m0 + m < words) {
-        float x[PER], y[PER];
-        cert_vec<DT>(q, m0 + m, x);
-        cert_vec<DT>(b, m0 + m, y);
-#pragma unroll
-        for (int e = 0; e < PER; ++e) {
-          const float t = __fsub_rn(x[e], y[e]);
-          p[m * PER + e] = __fmaf_rn(t, t, p[m * PER + e]);
-        }
-      }
-  }
-#pragma unroll
-  for (int s = 16; s >= 1; s >>= 1)
-#pragma unroll
-    for (int r = 0; r < s; ++r) p[r] = __fadd_rn(p[r], p[r + s]);
-  return p[0];
-}
 
 // One warp per sample.  The best screened entry gives a first canonical P; then
 // every column that the bound (k_screen.cu, certified exact scan) does not exclude
@@ -198,12 +288,13 @@ __device__ __forceinline__ float cert_dist(const void* q, const void* b, int d) 
 // whose screen gave up is listed instead.
 constexpr int kCertQueue = 8 + 32;  // a batch and the entries one part can add
 
-template <int DT>
+template <int DT, bool WIDE>
 __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A, int64_t nA, const int64_t* qidx,
                                                                const void* B, CertArgs c, float* min_d,
                                                                int64_t* argmin) {
   pdl_entry();
-  __shared__ int32_t s_queue[kRerankWarps][kCertQueue];
+  extern __shared__ __align__(16) float s_dyn[];  // the queries [warps][d]
+  __shared__ int32_t s_queue[kRerankWarps][kCertQueue], s_cols[kRerankWarps][32];
   const int lane = threadIdx.x & 31;
   int32_t* queue = s_queue[threadIdx.x >> 5];
   const int64_t l = int64_t(blockIdx.x) * kRerankWarps + (threadIdx.x >> 5);
@@ -232,12 +323,11 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
   const char* qrow = static_cast<const char*>(A) + size_t(a) * row_bytes;
   const size_t stride = size_t(c.T) * 32;  // entries of one part
   const size_t at = size_t(l) * 32 + lane;
+  float* q = s_dyn + size_t(threadIdx.x >> 5) * c.d;
+  stage_query<DT>(q, qrow, 1.0f, c.d, lane);
   // |q|^2, and the best entry over all parts (lane = class)
   float qn = 0.0f;
-  for (int j = lane; j < c.d; j += 32) {
-    const float x = load_elem<DT>(qrow, 0, c.d, j, nullptr);
-    qn = __fmaf_rn(x, x, qn);
-  }
+  for (int j = lane; j < c.d; j += 32) qn = __fmaf_rn(q[j], q[j], qn);
   float ms = __int_as_float(0x7F800000);
   int32_t mi = INT32_MAX;
 #pragma unroll 4
@@ -270,8 +360,17 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
   auto batch = [&](int cnt) {
     const int64_t b = lane < 4 * cnt ? int64_t(queue[lane >> 2]) + 32 * (lane & 3) : c.nB;
     float P = __int_as_float(0x7F800000);
+    if constexpr (WIDE) {
+      int32_t* cols = s_cols[threadIdx.x >> 5];
+      __syncwarp();
+      cols[lane] = static_cast<int32_t>(b < c.nB ? b : queue[0]);
+      __syncwarp();
+      const float v = group_dist<DT>(q, static_cast<const char*>(B), row_bytes, nullptr, cols, 4 * cnt, c.d);
+      if (b < c.nB) P = v;
+    } else if (b < c.nB) {
+      P = lane_dist<DT>(q, static_cast<const char*>(B) + size_t(b) * row_bytes, 1.0f, c.d);
+    }
     if (b < c.nB) {
-      P = cert_dist<DT>(qrow, static_cast<const char*>(B) + size_t(b) * row_bytes, c.d);
       const float dist = __fsqrt_rn(P);
       if (dist < best || (dist == best && static_cast<uint32_t>(b) < bidx)) {
         best = dist;
@@ -350,10 +449,14 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
 void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, const CertArgs& c, float* min_d,
                     int64_t* argmin, cudaStream_t s) {
   const int blocks = static_cast<int>(ceil_div(c.T, kRerankWarps));
-  if (A->dtype == CH_F32)
-    launch_k(k_certify<CH_F32>, blocks, 32 * kRerankWarps, 0, s, A->data, A->n, qidx, B->data, c, min_d, argmin);
-  else
-    launch_k(k_certify<CH_BF16>, blocks, 32 * kRerankWarps, 0, s, A->data, A->n, qidx, B->data, c, min_d, argmin);
+  auto run = [&](auto kern) {
+    CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRerankWarps * kMaxDim * 4));
+    launch_k(kern, blocks, 32 * kRerankWarps, size_t(kRerankWarps) * c.d * 4, s, A->data, A->n, qidx, B->data, c, min_d,
+             argmin);
+  };
+  const bool wide = size_t(c.d) * elem_size(A->dtype) >= kWideRow;
+  if (A->dtype == CH_F32) wide ? run(k_certify<CH_F32, true>) : run(k_certify<CH_F32, false>);
+  else wide ? run(k_certify<CH_BF16, true>) : run(k_certify<CH_BF16, false>);
   launch_check("certify");
 }
 
