@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(32 * kRerankWarps) k_rerank(const void* A, con
     if constexpr (WIDE) {
       if (n > 0) {
         int32_t* cols = s_cols[wib];
-        cols[lane] = col >= 0 ? col : first[0];
+        cols[lane] = col >= 0 ? col : 0;  // idle lanes read row 0 (an entry's own column may be past the end)
         __syncwarp();
         P = group_dist<DT>(q, static_cast<const char*>(B), row_bytes, scB, cols, 4 * n, d);
       }
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
     if constexpr (WIDE) {
       int32_t* cols = s_cols[threadIdx.x >> 5];
       __syncwarp();
-      cols[lane] = static_cast<int32_t>(b < c.nB ? b : queue[0]);
+      cols[lane] = static_cast<int32_t>(b < c.nB ? b : 0);
       __syncwarp();
       const float v = group_dist<DT>(q, static_cast<const char*>(B), row_bytes, nullptr, cols, 4 * cnt, c.d);
       if (b < c.nB) P = v;
