@@ -483,7 +483,8 @@ struct ScanBufs {
   ScanPart part;
   void* screen_work;
   int screen;
-  bool cert;  // the exact l2 scan runs in its certified tensor-core form
+  bool cert;   // the exact l2 scan runs in its certified tensor-core form
+  bool chain;  // the exact scan runs in its chained form
   float* norms;  // its |b|^2 where the set's own cannot be used
 };
 
@@ -501,11 +502,15 @@ static void take_scan(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, int64
   sb->screen = screen_choice(screen, metric, A, B);
   sb->cert = sb->screen == CH_SCREEN_EXACT && metric == CH_L2 && !plain && !c->exact_plain &&
              exact_tc_supported(A, B, T);
+  sb->chain = sb->screen == CH_SCREEN_EXACT && !sb->cert && !plain && !c->exact_plain && exact_chain_pays(A, B, T);
   if (sb->cert) {
     sb->part = ScanPart{nullptr, nullptr, 0, nullptr};
     sb->screen_work =
         lay.template take<char>(exact_tc_workspace(T, B->n, A->d, A->dtype, c->sm_count, c->screen_chunk_sms));
     sb->norms = norms_usable(c, B) ? nullptr : lay.template take<float>(size_t(B->n));
+  } else if (sb->chain) {
+    sb->part = ScanPart{nullptr, nullptr, 0, nullptr};
+    sb->screen_work = lay.template take<char>(exact_chain_workspace(T, B->n, c->sm_count));
   } else if (sb->screen == CH_SCREEN_EXACT) {
     sb->part.chunks = scan_exact_chunks(T, B->n, A->d, A->dtype, c->sm_count);
     sb->part.val = nullptr;
@@ -537,6 +542,10 @@ static void run_scan(ch_ctx* c, const ch_set* A, const int64_t* idx, int64_t T, 
     else ensure_norms(const_cast<ch_set*>(B), c->stream);
     launch_exact_tc(A, idx, T, B, sb->norms ? sb->norms : B->norms, sb->screen_work, m, argmin, c->sm_count,
                     c->screen_chunk_sms, c->stream, c->wait_cycles);
+    timer.stop(c->stream);
+  } else if (sb->chain) {
+    timer.start(c->stream);
+    launch_exact_chain(A, idx, T, B, metric, sb->screen_work, m, argmin, c->sm_count, c->stream);
     timer.stop(c->stream);
   } else if (sb->screen == CH_SCREEN_EXACT) {
     timer.start(c->stream);

@@ -16,6 +16,7 @@
 #include <cstring>
 
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/chamfer.h"
@@ -569,12 +570,20 @@ size_t exact_tc_workspace(int64_t T, int64_t nB, int d, int dtype, int sm_count,
 void launch_exact_tc(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const float* normB, void* work,
                      float* min_d, int64_t* argmin, int sm_count, int chunk_sms, cudaStream_t s, long long wait_cycles);
 
-// k_certify's part of it: samples l0 .. l0 + T - 1 with their screened classes
-// (part_* [parts][T][32]; part p covers chunk p / slices of B, columns
-// t * tile + (p % slices) * 128 + o * 32 + class, o < 4, of its tiles t)
+// The exact scan of d > 4 on CUDA cores in its chained form (k_chain.cu), for either
+// metric; the same minima and argmins, bit for bit.
+bool exact_chain_pays(const ch_set* A, const ch_set* B, int64_t T);
+size_t exact_chain_workspace(int64_t T, int64_t nB, int sm_count);
+void launch_exact_chain(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, void* work,
+                        float* min_d, int64_t* argmin, int sm_count, cudaStream_t s);
+
+// k_certify's part of both: samples l0 .. l0 + T - 1 with their classes (part_*
+// [parts][T][32]: smallest tile minimum, its first column, second smallest).  Part p
+// covers chunk p / slices of B, class c of it the columns t tile + (p % slices)
+// slice_cols + c class_cols + o occ_cols, o < 4, of the chunk's tiles t.
 struct CertArgs {
   int64_t l0, T, nB, chunk_len;
-  int d, parts, slices, tile;
+  int d, parts, slices, slice_cols, tile, class_cols, occ_cols;
   const float* part_s;
   const int32_t* part_i;
   const float* part_2;
@@ -584,10 +593,12 @@ struct CertArgs {
   uint32_t* ctl;            // [0] their number, [1] set when a screen gave up
   unsigned long long* best; // [T of the call] the list form's minima, set to all ones with each listing
 };
-void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, const CertArgs& c, float* min_d,
+void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, int metric, const CertArgs& c, float* min_d,
                     int64_t* argmin, cudaStream_t s);
+// dimensions the list form takes (the same as launch_scan_exact)
+bool scan_list_fits(int d);
 // the exact scan of the ctl[0] listed samples (at most T), written to their places
-void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const int32_t* list,
+void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, const int32_t* list,
                       const uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,
                       cudaStream_t s);
 

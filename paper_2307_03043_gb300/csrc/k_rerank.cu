@@ -37,8 +37,15 @@ __device__ __forceinline__ void stage_query(float* q, const char* row, float sc,
   __syncwarp();
 }
 
-// Squared canonical l2 distances of the staged row q to up to 32 rows of B.  Two forms,
-// the same sums in the same order:
+// p += |x - y| (l1) or (x - y)^2 (l2), rounded as the canonical distance rounds
+template <int METRIC>
+__device__ __forceinline__ void add_term(float& p, float x, float y) {
+  const float t = __fsub_rn(x, y);
+  p = METRIC == CH_L1 ? __fadd_rn(p, fabsf(t)) : __fmaf_rn(t, t, p);
+}
+
+// Canonical l1 sums or squared l2 distances of the staged row q to up to 32 rows of B.
+// Two forms for rows of a multiple of 16 bytes, the same sums in the same order:
 //  * lane_dist, rows below 512 bytes: a row per lane, the 32 partials in its registers,
 //    no shuffles; a warp keeps 32 rows in flight.  Its loads touch a sector per lane, so
 //    wide rows outgrow L1 between them;
@@ -51,7 +58,7 @@ __device__ __forceinline__ void stage_query(float* q, const char* row, float sc,
 // 256 / 97 / 94 us, fp8 d = 384 51 / - / 112 us.
 constexpr int kWideRow = 512;
 
-template <int DT>
+template <int DT, int METRIC>
 __device__ __forceinline__ float lane_dist(const float* __restrict__ q, const void* __restrict__ b, float sb, int d) {
   constexpr int PER = kRowPer<DT>;
   const int words = d / PER;
@@ -70,10 +77,7 @@ __device__ __forceinline__ float lane_dist(const float* __restrict__ q, const vo
           const float4 x = *reinterpret_cast<const float4*>(q + (m0 + m) * PER + e);
           const float xx[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float t = __fsub_rn(xx[k], y[e + k]);
-            p[m * PER + e + k] = __fmaf_rn(t, t, p[m * PER + e + k]);
-          }
+          for (int k = 0; k < 4; ++k) add_term<METRIC>(p[m * PER + e + k], xx[k], y[e + k]);
         }
       }
   }
@@ -86,7 +90,7 @@ __device__ __forceinline__ float lane_dist(const float* __restrict__ q, const vo
 
 // cols [32] in shared memory (entries from ncols on are ignored): the distance of row
 // cols[lane] on every lane < ncols
-template <int DT>
+template <int DT, int METRIC>
 __device__ __forceinline__ float group_dist(const float* __restrict__ q, const char* __restrict__ B, size_t row_bytes,
                                             const float* __restrict__ scB, const int32_t* cols, int ncols, int d) {
   constexpr int C = kRowPer<DT>, LPR = 32 / C, G = 32 / LPR, NR = DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1;
@@ -121,10 +125,7 @@ __device__ __forceinline__ float group_dist(const float* __restrict__ q, const c
         float y[C];
         row_vec<DT>(row[k], m, sb[k], y);
 #pragma unroll
-        for (int i = 0; i < C; ++i) {
-          const float t = __fsub_rn(x[i], y[i]);
-          p[k][i] = __fmaf_rn(t, t, p[k][i]);
-        }
+        for (int i = 0; i < C; ++i) add_term<METRIC>(p[k][i], x[i], y[i]);
       }
     }
 #pragma unroll
@@ -229,10 +230,10 @@ __global__ void __launch_bounds__(32 * kRerankWarps) k_rerank(const void* A, con
         int32_t* cols = s_cols[wib];
         cols[lane] = col >= 0 ? col : 0;  // idle lanes read row 0 (an entry's own column may be past the end)
         __syncwarp();
-        P = group_dist<DT>(q, static_cast<const char*>(B), row_bytes, scB, cols, 4 * n, d);
+        P = group_dist<DT, CH_L2>(q, static_cast<const char*>(B), row_bytes, scB, cols, 4 * n, d);
       }
     } else if (col >= 0) {
-      P = lane_dist<DT>(q, static_cast<const char*>(B) + size_t(col) * row_bytes, DT == CH_FP8E4M3 ? scB[col] : 1.0f, d);
+      P = lane_dist<DT, CH_L2>(q, static_cast<const char*>(B) + size_t(col) * row_bytes, DT == CH_FP8E4M3 ? scB[col] : 1.0f, d);
     }
     if (col >= 0) {
       const float dist = __fsqrt_rn(P);
@@ -288,13 +289,50 @@ namespace {
 // whose screen gave up is listed instead.
 constexpr int kCertQueue = 8 + 32;  // a batch and the entries one part can add
 
-template <int DT, bool WIDE>
-__global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A, int64_t nA, const int64_t* qidx,
-                                                               const void* B, CertArgs c, float* min_d,
-                                                               int64_t* argmin) {
+// FORM: how a batch's distances are formed.
+enum : int { CF_LANE = 0, CF_GROUP = 1, CF_ROWS = 2 };
+
+// CF_ROWS, for rows of any length: four rows at a time, lane r summing coordinates
+// j = r mod 32 of each, the tree by shuffles; cols as for group_dist
+template <int DT, int METRIC>
+__device__ __forceinline__ float rows_dist(const float* __restrict__ q, const void* __restrict__ B,
+                                           const float* __restrict__ scB, const int32_t* cols, int ncols, int d) {
+  const int lane = threadIdx.x & 31;
+  float mine = 0.0f;
+  for (int base = 0; base < ncols; base += 4) {
+    int64_t b[4];
+    float p[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      b[o] = cols[base + o < ncols ? base + o : 0];
+      p[o] = 0.0f;
+    }
+#pragma unroll 4
+    for (int j = lane; j < d; j += 32) {
+      const float x = q[j];
+#pragma unroll
+      for (int o = 0; o < 4; ++o) add_term<METRIC>(p[o], x, load_elem<DT>(B, b[o], d, j, scB));
+    }
+#pragma unroll
+    for (int sh = 16; sh >= 1; sh >>= 1)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) p[o] = __fadd_rn(p[o], __shfl_down_sync(0xFFFFFFFFu, p[o], sh));
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const float v = __shfl_sync(0xFFFFFFFFu, p[o], 0);
+      if (lane == base + o) mine = v;
+    }
+  }
+  return mine;
+}
+
+template <int DT, int METRIC, int FORM>
+__global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A, const float* scA, int64_t nA,
+                                                                  const int64_t* qidx, const void* B, const float* scB,
+                                                                  CertArgs c, float* min_d, int64_t* argmin) {
   pdl_entry();
   extern __shared__ __align__(16) float s_dyn[];  // the queries [warps][d]
-  __shared__ int32_t s_queue[kRerankWarps][kCertQueue], s_cols[kRerankWarps][32];
+  __shared__ int32_t s_queue[kRerankWarps][kCertQueue], s_cols[FORM != CF_LANE ? kRerankWarps : 1][32];
   const int lane = threadIdx.x & 31;
   int32_t* queue = s_queue[threadIdx.x >> 5];
   const int64_t l = int64_t(blockIdx.x) * kRerankWarps + (threadIdx.x >> 5);
@@ -319,15 +357,20 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
     give_up();
     return;
   }
-  const size_t row_bytes = size_t(c.d) * (DT == CH_F32 ? 4 : 2);
-  const char* qrow = static_cast<const char*>(A) + size_t(a) * row_bytes;
+  const size_t row_bytes = size_t(c.d) * (DT == CH_F32 ? 4 : DT == CH_BF16 ? 2 : 1);
   const size_t stride = size_t(c.T) * 32;  // entries of one part
   const size_t at = size_t(l) * 32 + lane;
-  float* q = s_dyn + size_t(threadIdx.x >> 5) * c.d;
-  stage_query<DT>(q, qrow, 1.0f, c.d, lane);
-  // |q|^2, and the best entry over all parts (lane = class)
+  float* q = s_dyn + size_t(threadIdx.x >> 5) * ((c.d + 3) / 4 * 4);
+  if constexpr (FORM == CF_ROWS) {
+    for (int j = lane; j < c.d; j += 32) q[j] = load_elem<DT>(A, a, c.d, j, scA);
+    __syncwarp();
+  } else {
+    stage_query<DT>(q, static_cast<const char*>(A) + size_t(a) * row_bytes, DT == CH_FP8E4M3 ? scA[a] : 1.0f, c.d, lane);
+  }
+  // |q|^2 where the threshold has a share of it, and the best entry over all parts (lane = class)
   float qn = 0.0f;
-  for (int j = lane; j < c.d; j += 32) qn = __fmaf_rn(q[j], q[j], qn);
+  if (c.q_scale != 0.0)
+    for (int j = lane; j < c.d; j += 32) qn = __fmaf_rn(q[j], q[j], qn);
   float ms = __int_as_float(0x7F800000);
   int32_t mi = INT32_MAX;
 #pragma unroll 4
@@ -356,22 +399,25 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
   float best = __int_as_float(0x7F800000);  // this lane's minimum and its column
   uint32_t bidx = 0xFFFFFFFFu;
   float bestP = best, thr = best;           // the warp's smallest squared distance, and its threshold
-  // queue[0 .. cnt - 1], cnt <= 8: lane 4 e + o takes column queue[e] + 32 o
+  // queue[0 .. cnt - 1], cnt <= 8: lane 4 e + o takes column queue[e] + o occ_cols
   auto batch = [&](int cnt) {
-    const int64_t b = lane < 4 * cnt ? int64_t(queue[lane >> 2]) + 32 * (lane & 3) : c.nB;
+    const int64_t b = lane < 4 * cnt ? int64_t(queue[lane >> 2]) + c.occ_cols * (lane & 3) : c.nB;
     float P = __int_as_float(0x7F800000);
-    if constexpr (WIDE) {
+    if constexpr (FORM != CF_LANE) {
       int32_t* cols = s_cols[threadIdx.x >> 5];
       __syncwarp();
       cols[lane] = static_cast<int32_t>(b < c.nB ? b : 0);
       __syncwarp();
-      const float v = group_dist<DT>(q, static_cast<const char*>(B), row_bytes, nullptr, cols, 4 * cnt, c.d);
+      const float v = FORM == CF_GROUP
+                          ? group_dist<DT, METRIC>(q, static_cast<const char*>(B), row_bytes, scB, cols, 4 * cnt, c.d)
+                          : rows_dist<DT, METRIC>(q, B, scB, cols, 4 * cnt, c.d);
       if (b < c.nB) P = v;
     } else if (b < c.nB) {
-      P = lane_dist<DT>(q, static_cast<const char*>(B) + size_t(b) * row_bytes, 1.0f, c.d);
+      P = lane_dist<DT, METRIC>(q, static_cast<const char*>(B) + size_t(b) * row_bytes,
+                                DT == CH_FP8E4M3 ? scB[b] : 1.0f, c.d);
     }
     if (b < c.nB) {
-      const float dist = __fsqrt_rn(P);
+      const float dist = METRIC == CH_L1 ? P : __fsqrt_rn(P);
       if (dist < best || (dist == best && static_cast<uint32_t>(b) < bidx)) {
         best = dist;
         bidx = static_cast<uint32_t>(b);
@@ -425,7 +471,8 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
     n += __popc(one);
     drain(7);
     for (unsigned rest = all; rest; rest &= rest - 1) {
-      const int64_t c0 = int64_t(p / c.slices) * c.chunk_len + (p % c.slices) * 128 + (__ffs(rest) - 1);
+      const int64_t c0 =
+          int64_t(p / c.slices) * c.chunk_len + (p % c.slices) * c.slice_cols + (__ffs(rest) - 1) * c.class_cols;
       const int64_t end = min(c.nB, (int64_t(p / c.slices) + 1) * c.chunk_len);
       for (int64_t b = c0; b < end; b += 32 * int64_t(c.tile)) {  // 32 tiles of the class at a time
         const int64_t mb = b + int64_t(lane) * c.tile;
@@ -446,17 +493,28 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
 
 }  // namespace
 
-void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, const CertArgs& c, float* min_d,
+void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, int metric, const CertArgs& c, float* min_d,
                     int64_t* argmin, cudaStream_t s) {
   const int blocks = static_cast<int>(ceil_div(c.T, kRerankWarps));
+  const size_t row = size_t(c.d) * elem_size(A->dtype);
+  const bool aligned = row % 16 == 0 && !((reinterpret_cast<uintptr_t>(A->data) | reinterpret_cast<uintptr_t>(B->data)) & 15);
   auto run = [&](auto kern) {
     CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRerankWarps * kMaxDim * 4));
-    launch_k(kern, blocks, 32 * kRerankWarps, size_t(kRerankWarps) * c.d * 4, s, A->data, A->n, qidx, B->data, c, min_d,
-             argmin);
+    launch_k(kern, blocks, 32 * kRerankWarps, size_t(kRerankWarps) * ((c.d + 3) / 4 * 4) * 4, s, A->data, A->scales, A->n,
+             qidx, B->data, B->scales, c, min_d, argmin);
   };
-  const bool wide = size_t(c.d) * elem_size(A->dtype) >= kWideRow;
-  if (A->dtype == CH_F32) wide ? run(k_certify<CH_F32, true>) : run(k_certify<CH_F32, false>);
-  else wide ? run(k_certify<CH_BF16, true>) : run(k_certify<CH_BF16, false>);
+  auto form = [&](auto dt, auto m) {
+    constexpr int DT = decltype(dt)::value, METRIC = decltype(m)::value;
+    if (!aligned) run(k_certify<DT, METRIC, CF_ROWS>);
+    else if (row >= kWideRow) run(k_certify<DT, METRIC, CF_GROUP>);
+    else run(k_certify<DT, METRIC, CF_LANE>);
+  };
+  auto go = [&](auto dt) {
+    metric == CH_L1 ? form(dt, std::integral_constant<int, CH_L1>{}) : form(dt, std::integral_constant<int, CH_L2>{});
+  };
+  if (A->dtype == CH_F32) go(std::integral_constant<int, CH_F32>{});
+  else if (A->dtype == CH_BF16) go(std::integral_constant<int, CH_BF16>{});
+  else go(std::integral_constant<int, CH_FP8E4M3>{});
   launch_check("certify");
 }
 

@@ -707,6 +707,8 @@ static size_t scan_smem(int d, bool db) {
   return size_t(d) * ((t.QT + 4) + (db ? 2 : 1) * (t.BT * t.SUB + 4)) * sizeof(float);
 }
 
+bool scan_list_fits(int d) { return scan_smem(d, false) <= 220 * 1024; }
+
 // Blocks of k_scan_exact one SM holds at once for dimension d: the dynamic
 // tiles, the static per-row minima (16 thread rows x QT x (4 + 8) bytes) and
 // the 1 KB reserved per block, out of 228 KB of shared memory per SM.
@@ -751,7 +753,9 @@ static void scan_launch(const ch_set* A, const int64_t* qidx, int64_t T, const c
   CHX_CHECK(tile_for(A->d).BT == BT && tile_for(A->d).SUB == SUB, CH_ENOTSUP, "scan tile mismatch");
   const size_t smem = scan_smem(A->d, db);
   if (list.list) {
-    if constexpr (METRIC == CH_L2 && DT != CH_FP8E4M3) {
+    // the two-sided instantiations would double the build: l1 and FP8 samples, which the
+    // chained scan hardly ever leaves over, take the forms with runtime loops
+    if constexpr ((METRIC == CH_L2 && DT != CH_FP8E4M3) || NJ == 0) {
       auto kern = k_scan_exact<DT, METRIC, QT, BT, PQ, PB, NJ, SUB, kDB, true>;
       CHX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
       launch_k(kern, part.chunks * scan_blocks_per_sm(A->d, db), 256, smem, s, A->data, A->scales, qidx, T, A->n,
@@ -772,7 +776,10 @@ template <int DT, int METRIC>
 static void scan_shape(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, ScanPart part,
                        cudaStream_t s, const ScanList& list = ScanList{nullptr, nullptr, nullptr}) {
   const TileShape t = tile_for(A->d);
-  if (A->d <= 128) {  // terms per partial fixed at compile time
+  constexpr bool kListNJ = METRIC == CH_L2 && DT != CH_FP8E4M3;
+  if (list.list && !kListNJ && A->d <= 32) {
+    scan_launch<DT, METRIC, 32, 64, 2, 4, 0, 4>(A, qidx, T, B, part, s, list);
+  } else if (A->d <= 128 && (!list.list || kListNJ)) {  // terms per partial fixed at compile time
     switch ((A->d + 31) / 32) {
       case 1: scan_launch<DT, METRIC, 32, 64, 2, 4, 1, 4>(A, qidx, T, B, part, s, list); break;
       case 2: scan_launch<DT, METRIC, 32, 64, 2, 4, 2>(A, qidx, T, B, part, s, list); break;
@@ -831,7 +838,7 @@ void launch_scan_exact(const ch_set* A, const int64_t* qidx, int64_t T, const ch
                        int sm_count, cudaStream_t s) {
   (void)sm_count;
   if (T == 0) return;
-  CHX_CHECK(scan_smem(A->d, false) <= 220 * 1024, CH_ENOTSUP, "dimension too large for the exact scan");
+  CHX_CHECK(scan_list_fits(A->d), CH_ENOTSUP, "dimension too large for the exact scan");
   switch (A->dtype) {
     case CH_F32: scan_metric<CH_F32>(A, qidx, T, B, metric, part, s); break;
     case CH_BF16: scan_metric<CH_BF16>(A, qidx, T, B, metric, part, s); break;
@@ -856,16 +863,18 @@ void launch_scan_merge(ScanPart part, int64_t T, int64_t nB, const int64_t* qidx
   launch_check("scan_merge");
 }
 
-void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, const int32_t* list,
+void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, const int32_t* list,
                       const uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,
                       cudaStream_t s) {
-  CHX_CHECK(scan_smem(A->d, false) <= 220 * 1024, CH_ENOTSUP, "dimension too large for the exact scan");
   const ScanList sl{list, ctl, best};
   const ScanPart grid{nullptr, nullptr, sm_count, nullptr};  // the list form's grid: sm_count x resident blocks
-  if (A->dtype == CH_F32)
-    scan_shape<CH_F32, CH_L2>(A, qidx, T, B, grid, s, sl);
-  else
-    scan_shape<CH_BF16, CH_L2>(A, qidx, T, B, grid, s, sl);
+  auto go = [&](auto dt) {
+    constexpr int DT = decltype(dt)::value;
+    metric == CH_L1 ? scan_shape<DT, CH_L1>(A, qidx, T, B, grid, s, sl) : scan_shape<DT, CH_L2>(A, qidx, T, B, grid, s, sl);
+  };
+  if (A->dtype == CH_F32) go(std::integral_constant<int, CH_F32>{});
+  else if (A->dtype == CH_BF16) go(std::integral_constant<int, CH_BF16>{});
+  else go(std::integral_constant<int, CH_FP8E4M3>{});
   launch_check("scan_list");
   launch_k(k_scan_list_out, static_cast<int>(std::min<int64_t>(ceil_div(T, 256), sm_count)), 256, 0, s, sl, min_d,
            argmin);

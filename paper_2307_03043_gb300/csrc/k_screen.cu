@@ -739,12 +739,17 @@ void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
 // candidates) whatever |A| is; 128 sample tiles still fill the SMs
 constexpr int64_t kCertSlice = 16384;
 
+// From 128 samples (a whole tile) and 2^20 pairs on, 2^23 below 512 samples, whose few
+// tiles leave SMs idle (k_scan_exact / certified: 1024 x 1024, d = 16 31 / 27 us; 512 x
+// 2048, d = 128 34.5 / 32.5 us; 2048 x 2048, d = 32 41 / 34 us; 256 x 4096, d = 64 22 / 39
+// us; 20k x 30k, d = 128 7.26 ms / 0.45 ms).
 bool exact_tc_supported(const ch_set* A, const ch_set* B, int64_t T) {
   if (A->dtype != B->dtype || (A->dtype != CH_F32 && A->dtype != CH_BF16)) return false;
   const int64_t row = int64_t(A->d) * int64_t(elem_size(A->dtype));
   if (A->d <= 4 || row % 16 != 0 || row > 16384) return false;
   if ((reinterpret_cast<uintptr_t>(A->data) & 15) || (reinterpret_cast<uintptr_t>(B->data) & 15)) return false;
-  return T >= 1 && B->n >= kBN && B->n < (int64_t(1) << 31) && T * B->n >= (int64_t(1) << 20);
+  return T >= kBM && B->n >= kBN && B->n < (int64_t(1) << 31) && T * B->n >= int64_t(T >= 512 ? 1 << 20 : 1 << 23) &&
+         scan_list_fits(A->d);
 }
 
 static int cert_screen(int dtype) { return dtype == CH_F32 ? CH_SCREEN_TF32 : CH_SCREEN_BF16; }
@@ -844,11 +849,14 @@ void launch_exact_tc(const ch_set* A, const int64_t* qidx, int64_t T, const ch_s
     c.part_2 = a.part_2;
     c.parts = kSlices * p.chunks;
     c.slices = kSlices;
+    c.slice_cols = kSliceCols;
     c.chunk_len = p.chunk_len;
     c.tile = kBN;
-    launch_certify(A, qidx, B, c, min_d, argmin, s);
+    c.class_cols = 1;
+    c.occ_cols = kClasses;
+    launch_certify(A, qidx, B, CH_L2, c, min_d, argmin, s);
   }
-  launch_scan_list(A, qidx, T, B, list, ctl, best, min_d, argmin, sm_count, s);
+  launch_scan_list(A, qidx, T, B, CH_L2, list, ctl, best, min_d, argmin, sm_count, s);
 }
 
 }  // namespace chx

@@ -55,9 +55,9 @@ def _check(ctx, A, B, idx, dtype=ch.CH_F32, metric=ch.CH_L2):
 
 
 @pytest.mark.parametrize("dtype", [ch.CH_F32, ch.CH_BF16], ids=["f32", "bf16"])
-@pytest.mark.parametrize("nB,d,T", [(257, 8, 4200), (1000, 16, 1100), (5003, 24, 300), (2560, 32, 511),
-                                    (4099, 40, 300), (2049, 128, 640), (3001, 200, 400), (1537, 384, 700),
-                                    (1111, 768, 1000), (700, 1000, 1500)])
+@pytest.mark.parametrize("nB,d,T", [(257, 8, 4200), (1000, 16, 1100), (5003, 24, 600), (2560, 32, 520),
+                                    (4099, 40, 530), (2049, 128, 640), (3001, 200, 560), (1537, 384, 700),
+                                    (1111, 768, 1000), (700, 1000, 1500), (40000, 16, 256)])
 def test_certified_scan_shapes(ctx, dtype, nB, d, T):
     A, B = workloads.gaussian_mixture(900, nB, d, nB + d, clusters=5)
     idx = np.random.default_rng(d).integers(0, 900, T).astype(np.int64)
@@ -122,6 +122,57 @@ def test_small_d_scan_data(ctx, metric, d, case):
     _check(ctx, A, B, idx, metric=metric)
 
 
+@pytest.mark.parametrize("dtype", [ch.CH_F32, ch.CH_BF16], ids=["f32", "bf16"])
+@pytest.mark.parametrize("metric", [ch.CH_L1, ch.CH_L2], ids=["l1", "l2"])
+@pytest.mark.parametrize("nB,d,T", [(9000, 33, 1900), (1801, 300, 1000), (10007, 97, 560), (5003, 127, 900),
+                                    (2500, 50, 4400), (30000, 5, 3700)])
+def test_chained_scan_shapes(ctx, metric, dtype, nB, d, T):
+    """Rows the screen cannot read, and l1: the chained form's tiles, slabs and sample
+    block widths (both metrics at sizes past its rule)."""
+    A, B = workloads.gaussian_mixture(400, nB, d, nB + d, clusters=5)
+    idx = np.random.default_rng(d).integers(0, 400, T).astype(np.int64)
+    idx[3::29] = -1
+    _check(ctx, A, B, idx, dtype, metric)
+
+
+@pytest.mark.parametrize("case", ["duplicates", "all_equal", "offset", "tiny", "huge", "one_far", "queries_in_B"])
+def test_chained_scan_data(ctx, case):
+    A, B = workloads.gaussian_mixture(600, 3000, 32, 11, clusters=4)
+    if case == "duplicates":
+        B[1500:] = B[:1500]
+    elif case == "all_equal":
+        B[:] = B[7]
+    elif case == "offset":
+        A += 3000
+        B += 3000
+    elif case == "tiny":
+        A *= np.float32(1e-33)
+        B *= np.float32(1e-33)
+    elif case == "huge":  # l1 sums overflow for the far rows
+        with np.errstate(over="ignore"):
+            B[::2] *= np.float32(3e36)
+    elif case == "one_far":
+        B[17] *= np.float32(1e15)
+        A[5] *= np.float32(1e15)
+    elif case == "queries_in_B":
+        B[100:700] = A
+    idx = np.random.default_rng(1).integers(0, 600, 5700).astype(np.int64)
+    _check(ctx, A, B, idx, metric=ch.CH_L1)
+
+
+@pytest.mark.parametrize("metric,d", [(ch.CH_L1, 24), (ch.CH_L2, 27)])
+def test_chained_brute_force_over_slices(ctx, metric, d):
+    A, B = workloads.uniform(17000, 1400, d, 6)
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    sA, sB = ch.ch_set_create(ctx, dA, 2, 17000, d), ch.ch_set_create(ctx, dB, 2, 1400, d)
+    mins = torch.zeros(17000, device="cuda")
+    v = ch.ch_exact(ctx, sA, sB, metric, 0, mins)
+    vo, mo = oracle.exact_canonical(A, B, metric)
+    assert np.array_equal(mins.cpu().numpy(), mo) and abs(v / vo - 1) < 1e-12
+    ch.ch_set_destroy(sA)
+    ch.ch_set_destroy(sB)
+
+
 def test_certified_brute_force_over_slices(ctx):
     """More samples than one slice of the scan, in A's order (ch_exact)."""
     A, B = workloads.uniform(17000, 333, 12, 5)
@@ -139,7 +190,7 @@ def test_certified_scan_survives_a_stopped_screen(ctx):
     """A wait budget that runs out inside the screen leaves the samples to the
     CUDA-core form: the exact scan never times out."""
     A, B = workloads.gaussian_mixture(500, 20000, 64, 3, clusters=6)
-    idx = np.random.default_rng(2).integers(0, 500, 400).astype(np.int64)
+    idx = np.random.default_rng(2).integers(0, 500, 520).astype(np.int64)
     ch.ch_ctx_set_wait_cycles(ctx, 8)
     try:
         _check(ctx, A, B, idx)
