@@ -840,10 +840,16 @@ def main():
         os.path.join(ROOT, "MEASURED_PEAKS.json")) else {}
     sm_max = peaks.get("sm_max_mhz", 2070.0)
     flops = 2.0 * T * NB * DIM  # algorithmic: one multiply-add per (sample, b, coordinate)
-    if screen_used == ch.CH_SCREEN_EXACT:
+    if screen_used == ch.CH_SCREEN_EXACT and DTYPE != "fp8" and DIM * elem_bytes() % 16 == 0:
+        # the exact l2 scan's certified form: the screen's contraction, then canonical distances
+        peak = peaks.get("bf16_tflops", 1910.1) * (1.1 / 2.25 if DTYPE == "f32" else 1.0)
+        roof = {"bound": "tensor", "achieved": flops / (kern_avg / 1e3) / 1e12, "peak": peak, "unit": "TFLOP/s",
+                "traffic": None, "kernel": "certified exact scan (k_screen + k_certify, 2*T*nB*d flops)",
+                "peak_basis": "of measured: bf16_tflops (burst) x nominal operand-type ratio"}
+    elif screen_used == ch.CH_SCREEN_EXACT:
         peak = 152 * 128 * sm_max * 1e6 / 1e12  # FP32 lanes x max clock, Tinst/s
         roof = {"bound": "alu", "achieved": flops / (kern_avg / 1e3) / 1e12, "peak": peak, "unit": "Tinst/s",
-                "traffic": None, "kernel": "k_scan_exact (canonical fp32 distances on CUDA cores)",
+                "traffic": None, "kernel": "k_chain + k_certify (exact scan on CUDA cores)",
                 "peak_basis": "152 SMs x 128 FP32 lanes x sm_max_mhz (derived, not measured)"}
     else:
         bf16 = peaks.get("bf16_tflops", 1910.1)
