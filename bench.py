@@ -386,7 +386,7 @@ def run_batched(args, ch, ctx, torch, rank, local, world):
     sm_max = peaks.get("sm_max_mhz", 2070.0)
     ops = 2.0 * rep.T * nB_big * DIM
     if rep.screen == ch.CH_SCREEN_EXACT:
-        kname = "k_scan_small" if DIM <= 4 else "k_scan_exact"
+        kname = "k_scan_small" if DIM <= 4 else "k_chain"
         roof = {"bound": "alu", "achieved": ops / (np.median(kms) / 1e3) / 1e12,
                 "peak": 152 * 128 * sm_max * 1e6 / 1e12, "unit": "Tinst/s", "traffic": None,
                 "kernel": f"{kname} (canonical fp32 l2 scan) {pair}",
