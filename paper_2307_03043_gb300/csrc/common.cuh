@@ -595,8 +595,9 @@ struct CertArgs {
 };
 void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, int metric, const CertArgs& c, float* min_d,
                     int64_t* argmin, cudaStream_t s);
-// dimensions the list form takes (the same as launch_scan_exact)
-bool scan_list_fits(int d);
+// what the list form takes: the dimensions of launch_scan_exact, and sample numbers
+// that fit the list's 32-bit entries (k_certify lists samples by their number)
+bool scan_list_fits(int64_t T, int d);
 // the exact scan of the ctl[0] listed samples (at most T), written to their places
 void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, const int32_t* list,
                       const uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,

@@ -261,7 +261,7 @@ void chain_launch(const ch_set* A, const int64_t* qidx, int64_t l0, int64_t n, c
 // T = 64 x 50k, d = 128: 82 / 111 us; T = 4.6k x 100k, d = 64: 2.90 / 2.0 ms; T = 3k x
 // 20k, d = 300 bf16: 2.47 / 1.46 ms).
 bool exact_chain_pays(const ch_set* A, const ch_set* B, int64_t T) {
-  return A->d > 4 && A->dtype == B->dtype && T >= 512 && B->n < (int64_t(1) << 31) && scan_list_fits(A->d) &&
+  return A->d > 4 && A->dtype == B->dtype && T >= 512 && B->n < (int64_t(1) << 31) && scan_list_fits(T, A->d) &&
          double(T) * double(B->n) * A->d >= double(1 << 29);
 }
 

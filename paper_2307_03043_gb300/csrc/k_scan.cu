@@ -707,7 +707,9 @@ static size_t scan_smem(int d, bool db) {
   return size_t(d) * ((t.QT + 4) + (db ? 2 : 1) * (t.BT * t.SUB + 4)) * sizeof(float);
 }
 
-bool scan_list_fits(int d) { return scan_smem(d, false) <= 220 * 1024; }
+static bool scan_fits(int d) { return scan_smem(d, false) <= 220 * 1024; }
+
+bool scan_list_fits(int64_t T, int d) { return T < (int64_t(1) << 31) && scan_fits(d); }
 
 // Blocks of k_scan_exact one SM holds at once for dimension d: the dynamic
 // tiles, the static per-row minima (16 thread rows x QT x (4 + 8) bytes) and
@@ -838,7 +840,7 @@ void launch_scan_exact(const ch_set* A, const int64_t* qidx, int64_t T, const ch
                        int sm_count, cudaStream_t s) {
   (void)sm_count;
   if (T == 0) return;
-  CHX_CHECK(scan_list_fits(A->d), CH_ENOTSUP, "dimension too large for the exact scan");
+  CHX_CHECK(scan_fits(A->d), CH_ENOTSUP, "dimension too large for the exact scan");
   switch (A->dtype) {
     case CH_F32: scan_metric<CH_F32>(A, qidx, T, B, metric, part, s); break;
     case CH_BF16: scan_metric<CH_BF16>(A, qidx, T, B, metric, part, s); break;

@@ -749,7 +749,7 @@ bool exact_tc_supported(const ch_set* A, const ch_set* B, int64_t T) {
   if (A->d <= 4 || row % 16 != 0 || row > 16384) return false;
   if ((reinterpret_cast<uintptr_t>(A->data) & 15) || (reinterpret_cast<uintptr_t>(B->data) & 15)) return false;
   return T >= kBM && B->n >= kBN && B->n < (int64_t(1) << 31) && T * B->n >= int64_t(T >= 512 ? 1 << 20 : 1 << 23) &&
-         scan_list_fits(A->d);
+         scan_list_fits(T, A->d);
 }
 
 static int cert_screen(int dtype) { return dtype == CH_F32 ? CH_SCREEN_TF32 : CH_SCREEN_BF16; }
