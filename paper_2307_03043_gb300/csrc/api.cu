@@ -244,6 +244,7 @@ static void run_hashed_pair(ch_ctx* c, const ch_set* A, const ch_set* B, const c
   hB->box_parts = launch_project(B, hp->hash_seed, k, hB->Y, hB->boxY, status, c->sm_count - half, c->side);
   CHX_CUDA(cudaEventRecord(c->join_ev, c->side));
   CHX_CUDA(cudaStreamWaitEvent(c->stream, c->join_ev, 0));
+  if (B->norms_on == c->side) const_cast<ch_set*>(B)->norms_on = c->stream;  // joined
 }
 
 template <class L>
@@ -488,12 +489,24 @@ struct ScanBufs {
   float* norms;  // its |b|^2 where the set's own cannot be used
 };
 
-// The exact l2 scan on c's stream can use the set's own |x|^2: the set belongs to c
-// (its lazy pass runs on c's stream, or c's parent's, which c's is ordered after) or
-// was prepared by a call that has returned.  Otherwise the scan makes its own: it
-// never wrote to another context's set, which others may be reading.
+// The exact l2 scan on c's stream can use the set's own |x|^2: a pass that has finished
+// (ch_set_prepare), one ordered before c's work (on c's stream, or on its parent's, after
+// which a lane's runs), or one that it runs itself on a set of its own.  A pass that any
+// other context enqueued (an asynchronous call may have, on a set of c's too) may still be
+// writing, and a captured one has not run: the scan then makes its own.
 static bool norms_usable(const ch_ctx* c, const ch_set* X) {
-  return X->ctx == c || X->ctx == c->parent || ((X->ready & READY_NORMS) && (X->ready & READY_SYNCED));
+  if (X->ready & READY_NORMS_DONE) return true;
+  if (capturing(c->stream)) return false;
+  if (!(X->ready & READY_NORMS)) return X->ctx == c;
+  return X->norms_on == c->stream || (c->parent && X->norms_on == c->parent->stream);
+}
+
+// the norms of X, if their pass has been enqueued, are finished once this returns; c's
+// stream has been synchronised
+static void settle_norms(ch_ctx* c, ch_set* X) {
+  if (!(X->ready & READY_NORMS) || (X->ready & READY_NORMS_DONE)) return;
+  if (X->norms_on != c->stream) CHX_CUDA(cudaDeviceSynchronize());  // another context's pass
+  X->ready |= READY_NORMS_DONE;
 }
 
 template <class L>
@@ -825,7 +838,7 @@ ch_status ch_set_embed(ch_ctx* c, ch_set* X, const ch_hash_params* hp) {
   launch_k(k_collect, 1, 32, 0, s, res, X->status, nullptr, nullptr, nullptr, nullptr, nullptr);
   launch_check("collect");
   finish(c, res, static_cast<ResBlock*>(c->host_pin));
-  X->ready |= READY_SYNCED;
+  settle_norms(c, X);
   X->hs.seed = hp->hash_seed;
   X->hs.k = k;
   X->hs.valid = true;
@@ -847,7 +860,7 @@ ch_status ch_set_prepare(ch_ctx* c, ch_set* X) {
   launch_k(k_collect, 1, 32, 0, s, res, X->status, nullptr, nullptr, nullptr, nullptr, nullptr);
   launch_check("collect");
   finish(c, res, static_cast<ResBlock*>(c->host_pin));
-  X->ready |= READY_SYNCED;
+  settle_norms(c, X);
   return CH_OK;
   CHX_GUARD_END
 }

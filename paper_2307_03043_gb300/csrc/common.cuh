@@ -156,15 +156,18 @@ struct ch_set {
   uint32_t* status = nullptr;  // device status word (ST_* bits)
   uint32_t* box_x = nullptr;   // ordered-encoded [2][d] bounding box of x (l1 hashed space)
   chx_hashed hs;               // cached l2 embedding
-  uint32_t ready = 0;          // READY_* passes already enqueued on the context's stream
+  uint32_t ready = 0;          // READY_* passes already enqueued
+  cudaStream_t norms_on = nullptr;  // the stream the norms pass is ordered on (READY_NORMS)
 };
 
 namespace chx {
 enum : uint32_t {
   READY_BOX_X = 1u << 0,  // box_x computed (and the finite check done)
   READY_NORMS = 1u << 1,  // norms computed (and the finite check done)
-  READY_SYNCED = 1u << 2,  // the passes above have finished on the device (ch_set_prepare, ch_set_embed)
+  READY_NORMS_DONE = 1u << 2,  // norms computed and finished on the device (ch_set_prepare, ch_set_embed)
 };
+// whether work on s runs only when a graph that is being captured is launched
+bool capturing(cudaStream_t s);
 // ingest pass (box of x, finite check) unless already done
 void ensure_ingest(ch_set* X, cudaStream_t s);
 // |x|^2 per row (sequential fmaf chain over j) unless already done

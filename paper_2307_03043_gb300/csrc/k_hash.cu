@@ -196,6 +196,13 @@ __global__ void __launch_bounds__(64) k_norms(const void* X, const float* scales
   if (status && __any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, ST_NONFINITE);
 }
 
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream beside a capture: not usable now
+  return true;
+}
+
 void launch_norms(const ch_set* X, float* norms, uint32_t* status, cudaStream_t s) {
   if (X->n == 0) return;
   const int grid = static_cast<int>(ceil_div(X->n, 64));
@@ -211,7 +218,10 @@ void launch_norms(const ch_set* X, float* norms, uint32_t* status, cudaStream_t 
 
 void ensure_norms(ch_set* X, cudaStream_t s) {
   if (X->ready & READY_NORMS) return;
-  X->ready |= READY_NORMS;
+  if (!capturing(s)) {
+    X->ready |= READY_NORMS;
+    X->norms_on = s;
+  }
   launch_norms(X, X->norms, X->status, s);
 }
 
@@ -1056,7 +1066,10 @@ int launch_project(const ch_set* X, uint64_t seed, int k, float* Y, uint32_t* bo
   // the set's |x|^2 and finite check come for free with this pass
   ch_set* mut = const_cast<ch_set*>(X);
   float* norms = (X->ready & READY_NORMS) ? nullptr : X->norms;
-  if (norms) mut->ready |= READY_NORMS;  // no write when ready (sets may be shared by host threads)
+  if (norms && !capturing(s)) {  // no write when ready (sets may be shared by host threads)
+    mut->ready |= READY_NORMS;
+    mut->norms_on = s;
+  }
   if (X->n == 0) {  // an empty box
     CHX_CUDA(cudaMemsetAsync(box, 0xFF, size_t(k) * 4, s));
     CHX_CUDA(cudaMemsetAsync(box + k, 0, size_t(k) * 4, s));
