@@ -164,12 +164,14 @@ __device__ inline uint32_t slot_home(uint64_t key, uint32_t log_cap) {
 // first: only the lowest lane (the smallest b, since b grows with the lane)
 // touches the table, which keeps the coarse scales -- where most points share
 // a handful of buckets -- from serialising on one L2 line.
-template <bool MERGE = true>
-__device__ inline void table_insert(ulonglong2* tab, uint32_t log_cap, uint64_t key, int64_t b, uint32_t* status) {
-  if (MERGE) {  // equal keys of a warp: only the lowest lane (the smallest b) inserts
-    const unsigned peers = __match_any_sync(__activemask(), static_cast<unsigned long long>(key));
-    if ((threadIdx.x & 31) != __ffs(peers) - 1) return;
-  }
+// lanes: the warp's lanes that insert in this round of its loop, agreed on by all of
+// them (round_lanes).  Lanes merely found side by side here (__activemask) may be in
+// different rounds, where a lower lane can hold a larger b, and the smaller one would
+// be dropped.
+__device__ inline void table_insert(ulonglong2* tab, uint32_t log_cap, uint64_t key, int64_t b, unsigned lanes,
+                                    uint32_t* status) {
+  const unsigned peers = __match_any_sync(lanes, static_cast<unsigned long long>(key));
+  if ((threadIdx.x & 31) != __ffs(peers) - 1) return;
   const uint32_t cap = 1u << log_cap;
   const unsigned long long want = ~static_cast<unsigned long long>(b);
   uint32_t pos = slot_home(key, log_cap);
@@ -197,6 +199,10 @@ __device__ inline void table_insert(ulonglong2* tab, uint32_t log_cap, uint64_t 
   }
   atomicOr(status, ST_TABLE_FULL);
 }
+
+// The lanes whose row r of this round exists; the whole warp meets here each round
+// (0: none is left, and every lane leaves the loop).
+__device__ __forceinline__ unsigned round_lanes(int64_t r, int64_t n) { return __ballot_sync(0xFFFFFFFFu, r < n); }
 
 // bucket of key at one scale: the smallest b, or -1 if empty
 __device__ inline int64_t table_find(const ulonglong2* tab, uint32_t log_cap, uint64_t key) {
@@ -269,10 +275,12 @@ __global__ void __launch_bounds__(128) k_table_insert_ps(HashSrc src, int L, int
   load_group_consts(gc, t, src.dd, L, L0, nl);
   const int l = blockIdx.y;
   const size_t cap = size_t(1) << h.log_cap;
-  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < src.n; r += int64_t(gridDim.x) * blockDim.x) {
+  int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (unsigned lanes; (lanes = round_lanes(r, src.n)) != 0; r += int64_t(gridDim.x) * blockDim.x) {
+    if (r >= src.n) continue;
     float y[W];
     load_row<DT, W>(src, r, y);
-    table_insert(h.slots + size_t(l) * cap, h.log_cap, group_key(y, src.dd, l, gc), r, status);
+    table_insert(h.slots + size_t(l) * cap, h.log_cap, group_key(y, src.dd, l, gc), r, lanes, status);
   }
 }
 
@@ -282,14 +290,16 @@ __global__ void __launch_bounds__(128) k_table_insert(HashSrc src, int L, int L0
   pdl_entry();
   if (group_mode(h) != GM_FWD) return;
   const size_t cap = size_t(1) << h.log_cap;
-  for (int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; r < src.n; r += int64_t(gridDim.x) * blockDim.x) {
+  int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (unsigned lanes; (lanes = round_lanes(r, src.n)) != 0; r += int64_t(gridDim.x) * blockDim.x) {
+    if (r >= src.n) continue;
     for (int b0 = 0; b0 < nl; b0 += kLevelBlock) {
       uint64_t key[kLevelBlock];
       const int nb = min(kLevelBlock, nl - b0);
       stream_keys<DT>(src, r, L, L0 + b0, nb, t, key);
 #pragma unroll
       for (int l = 0; l < kLevelBlock; ++l)
-        if (l < nb) table_insert(h.slots + size_t(b0 + l) * cap, h.log_cap, key[l], r, status);
+        if (l < nb) table_insert(h.slots + size_t(b0 + l) * cap, h.log_cap, key[l], r, lanes, status);
     }
   }
 }
@@ -461,10 +471,12 @@ __global__ void __launch_bounds__(128) k_table_insert_batch(const CrudePair* P, 
   load_group_consts(gc, p.t, p.B.dd, p.L, 0, p.L);
   const HashSrc src = p.B;
   const size_t cap = size_t(1) << p.log_cap;
-  for (int64_t r = int64_t(local % gx) * blockDim.x + threadIdx.x; r < src.n; r += int64_t(gx) * blockDim.x) {
+  int64_t r = int64_t(local % gx) * blockDim.x + threadIdx.x;
+  for (unsigned lanes; (lanes = round_lanes(r, src.n)) != 0; r += int64_t(gx) * blockDim.x) {
+    if (r >= src.n) continue;
     float y[W];
     load_row<DT, W>(src, r, y);
-    table_insert(p.slots + size_t(l) * cap, p.log_cap, group_key(y, src.dd, l, gc), r, p.status);
+    table_insert(p.slots + size_t(l) * cap, p.log_cap, group_key(y, src.dd, l, gc), r, lanes, p.status);
   }
 }
 
