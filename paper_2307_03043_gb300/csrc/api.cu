@@ -65,34 +65,35 @@ struct Layout {
   }
 };
 
-// Where the workspace does not fit, the layout is taken again with the exact l2
-// scan in its CUDA-core form, which needs less scratch and gives the same bits.
+// f(layout, plain) takes the buffers of a call that may scan.  Where the workspace does
+// not fit (or with plain set), they are taken with the exact scan in its plain form,
+// which needs less scratch and gives the same bits.  The choice is a value handed
+// down, never kept in the context: other threads size requests by it (serve.cu).
 template <class F>
-static void carve(ch_ctx* c, F&& f) {
-  struct Restore {
-    ch_ctx* c;
-    bool was;
-    ~Restore() { c->exact_plain = was; }
-  } restore{c, c->exact_plain};
+static void carve_scan(ch_ctx* c, F&& f, bool plain = false) {
   Layout m;
-  f(m);
+  f(m, plain);
   try {
     c->ws.reserve(m.need + 256);
   } catch (const Err& e) {
-    if (e.st != CH_ENOMEM || c->exact_plain) throw;
-    c->exact_plain = true;
-    Layout plain;
-    f(plain);
-    if (plain.need >= m.need) throw;
-    c->ws.reserve(plain.need + 256);
+    if (e.st != CH_ENOMEM || plain) throw;
+    plain = true;
+    Layout p;
+    f(p, plain);
+    if (p.need >= m.need) throw;
+    c->ws.reserve(p.need + 256);
   }
   c->ws.reset();
   Layout t;
   t.measure = false;
   t.a = &c->ws;
-  f(t);
+  f(t, plain);
 }
 
+template <class F>
+static void carve(ch_ctx* c, F&& f) {
+  carve_scan(c, [&](auto& lay, bool) { f(lay); }, true);
+}
 
 __global__ void k_collect(ResBlock* r, const uint32_t* sa, const uint32_t* sb, const double* out2,
                           const uint64_t* W, const int32_t* S, const int32_t* e_top) {
@@ -511,11 +512,10 @@ static void settle_norms(ch_ctx* c, ch_set* X) {
 
 template <class L>
 static void take_scan(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, int64_t T, int metric, int screen,
-                      uint32_t R, ScanBufs* sb, bool plain = false) {
+                      uint32_t R, ScanBufs* sb, bool plain) {
   sb->screen = screen_choice(screen, metric, A, B);
-  sb->cert = sb->screen == CH_SCREEN_EXACT && metric == CH_L2 && !plain && !c->exact_plain &&
-             exact_tc_supported(A, B, T);
-  sb->chain = sb->screen == CH_SCREEN_EXACT && !sb->cert && !plain && !c->exact_plain && exact_chain_pays(A, B, T);
+  sb->cert = sb->screen == CH_SCREEN_EXACT && metric == CH_L2 && !plain && exact_tc_supported(A, B, T);
+  sb->chain = sb->screen == CH_SCREEN_EXACT && !sb->cert && !plain && exact_chain_pays(A, B, T);
   if (sb->cert) {
     sb->part = ScanPart{nullptr, nullptr, 0, nullptr};
     sb->screen_work =
@@ -592,7 +592,7 @@ struct EstBufs {
 
 template <class L>
 static void take_estimate(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p, int64_t T,
-                          uint32_t R, EstBufs* eb, bool plain = false) {
+                          uint32_t R, EstBufs* eb, bool plain) {
   const int64_t nA = A->n;
   eb->res = lay.template take<ResBlock>(1);
   eb->out2 = lay.template take<double>(kCombineDoubles);
@@ -608,7 +608,8 @@ static void take_estimate(L& lay, ch_ctx* c, const ch_set* A, const ch_set* B, c
 }
 
 // device workspace bytes ch_estimate(A, B, p) needs on a context like c; with
-// plain, those of the CUDA-core form of the exact scan (what carve falls back to)
+// plain, those of the plain form of the exact scan (what carve_scan falls back to);
+// reads nothing of c that a call on it changes
 size_t estimate_footprint(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p, bool plain) {
   const uint32_t R = p->rerank_k ? p->rerank_k : 8;
   const int64_t T = p->T > 0 ? p->T : default_T(A->n, B->n, p->eps);
@@ -1007,9 +1008,9 @@ ch_status ch_sampled_nn(ch_ctx* c, const ch_set* A, const int64_t* idx, int64_t 
   CHX_CUDA(cudaSetDevice(c->device));
   ScanBufs sc;
   uint32_t* st = nullptr;
-  carve(c, [&](auto& lay) {
+  carve_scan(c, [&](auto& lay, bool plain) {
     st = lay.template take<uint32_t>(1);
-    take_scan(lay, c, A, B, T, metric, screen, rerank_k, &sc);
+    take_scan(lay, c, A, B, T, metric, screen, rerank_k, &sc, plain);
   });
   CHX_CUDA(cudaMemsetAsync(st, 0, 4, c->stream));
   run_scan(c, A, idx, T, B, metric, rerank_k, &sc, min_d, argmin, st);
@@ -1410,17 +1411,8 @@ static ResBlock* estimate_enqueue(ch_ctx* c, const ch_set* A, const ch_set* B, c
                                   uint32_t R, ResBlock* res_out, bool events, int* screen_used,
                                   ResBlock* host_out = nullptr, bool lone = false) {
   EstBufs eb;
-  carve(c, [&](auto& lay) { take_estimate(lay, c, A, B, p, T, R, &eb); });
+  carve_scan(c, [&](auto& lay, bool plain) { take_estimate(lay, c, A, B, p, T, R, &eb, plain); });
   return estimate_run(c, A, B, p, T, R, eb, res_out, events, screen_used, host_out, lone, false);
-}
-
-// the workspace bytes estimate_enqueue carves for (A, B, p)
-static size_t estimate_need(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_est_params* p, int64_t T,
-                            uint32_t R) {
-  Layout m;
-  EstBufs eb;
-  take_estimate(m, c, A, B, p, T, R, &eb);
-  return m.need + 256;
 }
 
 }  // namespace chx
@@ -1531,6 +1523,7 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
   std::vector<char> bcr(count, 0);
   for (int64_t i : run) bcr[i] = crude_batchable(A[i], B[i], &params[i]);
   std::vector<size_t> need(K, 0);
+  bool plain = false;  // every lane's exact scans keep to the plain form
   auto lane_needs = [&] {
     std::fill(need.begin(), need.end(), 0);
     for (int64_t i : run) {
@@ -1544,30 +1537,37 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
         mc.template take<uint8_t>(A[i]->n);  // level
       }
       ScanBufs sc;
-      if (!small[i]) take_scan(ms, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc);
+      if (!small[i]) take_scan(ms, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc, plain);
       need[i % K] = std::max(need[i % K], std::max(mc.need, ms.need) + 256);
     }
     for (int k = 0; k < K; ++k) c->lanes[k]->ws.reserve(need[k]);
   };
-  for (int k = 0; k < K; ++k) c->lanes[k]->exact_plain = false;
   try {
     lane_needs();
-  } catch (const Err& e) {  // the exact l2 scans' CUDA-core form needs less scratch (see carve)
+  } catch (const Err& e) {  // the plain form needs less scratch (see carve_scan)
     if (e.st != CH_ENOMEM) throw;
-    for (int k = 0; k < K; ++k) c->lanes[k]->exact_plain = true;
+    plain = true;
     lane_needs();
   }
   // the batch allocation: result blocks, the work list, then each pair's arrays
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   size_t arena = al(sizeof(ResBlock) * count) + al(sizeof(BatchItem) * std::max<size_t>(run.size(), 1));
-  size_t best_bytes = 0;  // the small pairs' minima (distance bits << 32), one block (cleared together)
+  size_t best_bytes = 0;  // the small pairs' minima (distance bits, index), one block (cleared together)
   for (int64_t i : run) {
     arena += al(size_t(A[i]->n) * 4) + 2 * al(size_t(A[i]->n) * 8) + al(size_t(Ts[i]) * 8) + al(size_t(Ts[i]) * 4);
     if (small[i]) best_bytes += al(size_t(Ts[i]) * 8);
   }
   arena += best_bytes;
   char* mem = nullptr;
-  CHX_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&mem), arena, c->pool, c->stream));
+  cudaError_t got = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&mem), arena, c->pool, c->stream);
+  if (got == cudaErrorMemoryAllocation && !plain) {  // the lanes' scratch may be what is in its way
+    cudaGetLastError();
+    plain = true;
+    for (int k = 0; k < K; ++k) c->lanes[k]->ws.release();
+    lane_needs();
+    got = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&mem), arena, c->pool, c->stream);
+  }
+  CHX_CUDA(got);
   ResBlock* dres = reinterpret_cast<ResBlock*>(mem);
   BatchItem* ditems = reinterpret_cast<BatchItem*>(mem + al(sizeof(ResBlock) * count));
   char* cur = mem + al(sizeof(ResBlock) * count) + al(sizeof(BatchItem) * std::max<size_t>(run.size(), 1));
@@ -1708,7 +1708,9 @@ ch_status ch_estimate_batch(ch_ctx* c, int64_t count, const ch_set* const* A, co
   on_lanes([&](int64_t i) { return !small[i]; }, [&](ch_ctx* lane, int64_t i) {
     const ch_est_params* p = &params[i];
     ScanBufs sc;
-    carve(lane, [&](auto& lay) { take_scan(lay, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc); });
+    carve_scan(lane, [&](auto& lay, bool pl) {
+      take_scan(lay, lane, A[i], B[i], Ts[i], p->hash.metric, p->screen, Rs[i], &sc, pl);
+    }, plain);
     run_scan(lane, A[i], idxp[i], Ts[i], B[i], p->hash.metric, Rs[i], &sc, mp[i], nullptr, &dres[i].status);
   });
   if (best_bytes) {
@@ -1788,9 +1790,9 @@ ch_status ch_estimate_sym(ch_ctx* c, const ch_set* A, const ch_set* B, const ch_
   check_estimate(c, B, A, &pb, &Tba, &Rb);
   CHX_CUDA(cudaSetDevice(c->device));
   EstBufs e1, e2;
-  carve(c, [&](auto& lay) {
-    take_estimate(lay, c, A, B, p, Tab, R, &e1);
-    take_estimate(lay, c, B, A, &pb, Tba, Rb, &e2);
+  carve_scan(c, [&](auto& lay, bool plain) {
+    take_estimate(lay, c, A, B, p, Tab, R, &e1, plain);
+    take_estimate(lay, c, B, A, &pb, Tba, Rb, &e2, plain);
   });
   ResBlock* h = static_cast<ResBlock*>(c->host_pin);  // [0]: (A, B), [1]: (B, A)
   estimate_run(c, A, B, p, Tab, R, e1, nullptr, false, nullptr, h, true, false);
@@ -1820,10 +1822,10 @@ ch_status ch_exact(ch_ctx* c, const ch_set* A, const ch_set* B, int32_t metric, 
   ResBlock* res = nullptr;
   float* mins = per_a_min;
   double* out2 = nullptr;
-  carve(c, [&](auto& lay) {
+  carve_scan(c, [&](auto& lay, bool plain) {
     res = lay.template take<ResBlock>(1);
     out2 = lay.template take<double>(kCombineDoubles);
-    take_scan(lay, c, A, B, nA, metric, mode == 0 ? CH_SCREEN_EXACT : CH_SCREEN_AUTO, 8, &sc);
+    take_scan(lay, c, A, B, nA, metric, mode == 0 ? CH_SCREEN_EXACT : CH_SCREEN_AUTO, 8, &sc, plain);
     float* tmp = lay.template take<float>(std::max<int64_t>(nA, 1));
     if (!per_a_min) mins = tmp;
   });

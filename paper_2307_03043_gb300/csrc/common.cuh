@@ -129,7 +129,6 @@ struct ch_ctx {
   bool own_stream = false;
   int sm_count = 0;
   int screen_chunk_sms = 0;  // SMs the screen's B split aims to fill (0: all); a batch lane's share
-  bool exact_plain = false;  // the exact l2 scan keeps to CUDA cores (a call whose certified form's scratch did not fit)
   long long wait_cycles = 0;  // budget of the tensor-core screen's pipeline waits, SM cycles (0: about 2 s)
   chx::Arena ws;
   cudaMemPool_t pool = nullptr;  // stream-ordered pool for sets; keeps freed memory
