@@ -8,7 +8,10 @@
 //    for its sizes and parameters; a scheduler thread admits queued requests in
 //    arrival order while a slot is free and the admitted footprints stay within
 //    the budget (sets excluded).  A request larger than the whole budget is
-//    refused at submission (CH_EBUSY).
+//    refused at submission (CH_EBUSY).  Exact scans run in one of two forms, the
+//    faster of which needs more scratch (an l1 request of T = 4.6k x 100k, d = 64:
+//    37 MB more); the plain one's footprint decides admission, and a request gets
+//    the faster form only where its scratch is in nobody's way (see fast_fits).
 //  * Each slot owns a context (stream) and a worker thread; an admitted
 //    request's workspace comes from the server's stream-ordered pool, so
 //    requests of different sizes overlap on the device without reallocations.
@@ -44,7 +47,8 @@ struct Request {
   uint64_t ticket = 0;
   uint64_t a = 0, b = 0;
   ch_est_params p{};
-  size_t footprint = 0;
+  size_t plain = 0, fast = 0;  // footprints of the exact scan's forms
+  size_t footprint = 0;        // the one it was admitted with
   Clock::time_point t_submit, t_done;
   bool done = false;
   ch_status status = CH_EAGAIN;
@@ -91,6 +95,20 @@ struct ch_server {
 
 namespace {
 
+// Whether the request about to be admitted (already off the queue, `free_slots` slots
+// left after it) may take its faster form: within an equal share of the budget, so
+// that requests alike fill every slot as they do in the plain form, and with room
+// left for the waiting requests that the remaining slots could run.
+bool fast_fits(const ch_server* s, const Request& r, int64_t free_slots) {
+  if (int64_t(r.fast) > s->cfg.hbm_budget_bytes / s->cfg.max_slots) return false;
+  int64_t need = s->in_use + int64_t(r.fast);
+  for (size_t i = 0; i < s->queue.size() && int64_t(i) < free_slots; ++i) {
+    if (need > s->cfg.hbm_budget_bytes) return false;
+    need += int64_t(s->queue[i]->plain);
+  }
+  return need <= s->cfg.hbm_budget_bytes;
+}
+
 void scheduler_loop(ch_server* s) {
   std::unique_lock<std::mutex> lk(s->mu);
   while (true) {
@@ -98,11 +116,13 @@ void scheduler_loop(ch_server* s) {
       if (s->stop) return true;
       if (s->queue.empty()) return false;
       const bool free_slot = std::any_of(s->slot_req.begin(), s->slot_req.end(), [](auto& r) { return !r; });
-      return free_slot && s->in_use + int64_t(s->queue.front()->footprint) <= s->cfg.hbm_budget_bytes;
+      return free_slot && s->in_use + int64_t(s->queue.front()->plain) <= s->cfg.hbm_budget_bytes;
     });
     if (s->stop) return;
     auto r = s->queue.front();
     s->queue.pop_front();
+    const int64_t free_slots = std::count(s->slot_req.begin(), s->slot_req.end(), nullptr) - 1;
+    r->footprint = fast_fits(s, *r, free_slots) ? r->fast : r->plain;
     for (size_t i = 0; i < s->slot_req.size(); ++i)
       if (!s->slot_req[i]) {
         s->slot_req[i] = r;
@@ -128,9 +148,9 @@ ch_status run_request(ch_server* s, ch_ctx* c, Request& r, double* eta) {
   if (cudaSetDevice(c->device) != cudaSuccess) return CH_ECUDA;
   size_t bytes = r.footprint;
   cudaError_t got = cudaMallocFromPoolAsync(&ws, bytes + 256, s->main->pool, c->stream);
-  if (got != cudaSuccess) {  // once more with the exact scan's CUDA-core form
+  if (got != cudaSuccess && bytes > r.plain) {  // once more with the exact scan's plain form
     cudaGetLastError();
-    bytes = std::min(bytes, chx::estimate_footprint(c, A, B, &r.p, true));
+    bytes = r.plain;
     got = cudaMallocFromPoolAsync(&ws, bytes + 256, s->main->pool, c->stream);
   }
   if (got != cudaSuccess) {
@@ -268,11 +288,9 @@ ch_status ch_serve_submit(ch_server* s, uint64_t setA, uint64_t setB, const ch_e
     const ch_set* B = ib->second;
     if (A->d != B->d || A->dtype != B->dtype || B->n < 1) return CH_EINVAL;
     if (p->T < 0 || (p->T == 0 && !(p->eps > 0.0 && p->eps < 1.0))) return CH_EINVAL;
-    r->footprint = chx::estimate_footprint(s->slot_ctx[0], A, B, p, false);
-    // a budget too small for the exact scan's tensor-core form gets its CUDA-core form
-    if (int64_t(r->footprint) > s->cfg.hbm_budget_bytes)
-      r->footprint = chx::estimate_footprint(s->slot_ctx[0], A, B, p, true);
-    if (s->fault == Fault::admit || int64_t(r->footprint) > s->cfg.hbm_budget_bytes) {
+    r->fast = chx::estimate_footprint(s->slot_ctx[0], A, B, p, false);
+    r->plain = std::min(r->fast, chx::estimate_footprint(s->slot_ctx[0], A, B, p, true));
+    if (s->fault == Fault::admit || int64_t(r->plain) > s->cfg.hbm_budget_bytes) {
       ++s->rejected;
       return CH_EBUSY;
     }
