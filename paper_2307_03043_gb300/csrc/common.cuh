@@ -526,6 +526,12 @@ int scan_small_segments(int64_t nB);
 void launch_scan_merge(ScanPart part, int64_t T, int64_t nB, const int64_t* qidx, float* min_d, int64_t* argmin,
                        cudaStream_t s);
 int scan_exact_chunks(int64_t T, int64_t nB, int d, int dtype, int sm_count);
+// the parts of both for d <= kScanSmallMaxD (k_small.cu)
+void launch_scan_small(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, ScanPart part,
+                       cudaStream_t s);
+void launch_scan_small_out(ScanPart part, int64_t T, int64_t nB, const int64_t* qidx, float* min_d, int64_t* argmin,
+                           cudaStream_t s);
+int scan_small_chunks(int64_t T, int64_t nB, int sm_count);
 
 // ---- batched exact scan of small dimensions (d <= 4) over many pairs at once
 constexpr int kBatchScanMaxD = 4;

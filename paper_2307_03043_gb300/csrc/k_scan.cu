@@ -9,8 +9,6 @@
 // leaves are all beyond d are +0 and skipped (adding +0 to a non-negative
 // partial is exact).  The result is bit-identical to the definition, for both
 // the minimum and the smallest-index argmin.
-#include <type_traits>
-
 #include "common.cuh"
 
 namespace chx {
@@ -321,347 +319,6 @@ __global__ void k_scan_list_out(ScanList sl, float* min_d, int64_t* argmin) {
   }
 }
 
-// Small dimensions (d <= 4, known at compile time): every partial p_r of the
-// canonical distance holds the single term of coordinate r, so the halving tree
-// reduces to a fixed expression, folded here at compile time.
-constexpr int kSmallMaxD = 4;
-constexpr int64_t kSmallSegment = int64_t(1) << 31;  // rows whose index fits best[]'s low word
-constexpr int kSmallBT = 1024;   // rows of B per shared-memory stage
-constexpr int kSmallSub = 32;    // rows per sub-tile: the unit the minima are tracked and evaluated in
-constexpr int kSmallPQ = 4;      // samples per thread of a lone scan
-constexpr int kSmallQ = 256 * kSmallPQ;
-constexpr int kBatchPQ = 8;      // most samples per thread of a batched scan
-
-// partial R after tree steps 16 .. S (S = 32: the leaf) for d = D <= 32 terms
-template <int D, int R, int S>
-__device__ __forceinline__ float small_node(const float (&leaf)[D]) {
-  if constexpr (S == 32) {
-    return leaf[R];
-  } else if constexpr (R + S < D) {
-    return __fadd_rn(small_node<D, R, 2 * S>(leaf), small_node<D, R + S, 2 * S>(leaf));
-  } else {
-    return small_node<D, R, 2 * S>(leaf);
-  }
-}
-
-// canonical l1 sum or squared l2 sum of q and b
-template <int METRIC, int D>
-__device__ __forceinline__ float small_canon(const float (&q)[D], const float (&b)[D]) {
-  float leaf[D];
-#pragma unroll
-  for (int j = 0; j < D; ++j) {
-    const float t = __fsub_rn(q[j], b[j]);
-    leaf[j] = (METRIC == CH_L1) ? fabsf(t) : __fmul_rn(t, t);
-  }
-  return small_node<D, 0, 1>(leaf);
-}
-
-// element j of row r, the storage type known at run time (the scans of d <= 4 spend
-// their time past the loads, and one instantiation serves every type)
-__device__ __forceinline__ float elem_of(int dtype, const void* base, int64_t r, int d, int j, const float* scales) {
-  return dtype == CH_F32    ? load_elem<CH_F32>(base, r, d, j, scales)
-         : dtype == CH_BF16 ? load_elem<CH_BF16>(base, r, d, j, scales)
-                            : load_elem<CH_FP8E4M3>(base, r, d, j, scales);
-}
-
-// 256 x PQ samples (l0 + thread + 256 p) against rows b_begin .. b_end - 1 of B; the
-// minimum (distance bits, index) of each folds into best[] by atomicMin.
-//
-// A thread keeps PQ samples in registers and walks a shared-memory stage of B two
-// rows at a time in packed f32x2 instructions (broadcast 16-byte reads), keeping only
-// each sample's smallest value per 32-row sub-tile and the sub-tiles that hold its
-// smallest ones; a warp then evaluates the canonical distance of the rows of the
-// sub-tiles that matter, a row per lane.
-//   l1: the value is the canonical sum itself (3 packed subtractions, 4 additions of
-//       |t| and one three-input minimum for two rows at d = 3); the first sub-tile
-//       with the smallest value holds the answer.
-//   l2: the value is L = |b|^2 shrink - 2 q.b (d packed fused multiply-adds for two
-//       rows, the norms staged with the rows) instead of the canonical 3 d - 1
-//       operations per row.  With u = 2^-24: the norm's chain is within d u |b|^2, the
-//       d fmas within 1.01 d u (|b|^2 + 2 |q||b|) and 2 |q||b| <= |q|^2 + |b|^2, so with
-//       shrink = 1 - 4 d u every row has |q - b|^2 >= L + |q|^2 (1 - 1.01 d u).  A row
-//       that ties with or beats a canonical squared distance P (itself within 10 u, and
-//       equal square roots within 2^-22) therefore has
-//         L <= P (1 + 2^-19) - |q|^2 (1 - (2.1 d + 2) u) + 2^-100.
-//       The best sub-tile gives P; the second is evaluated where it meets this, the
-//       whole chunk where the third does (or where magnitudes leave the bound's range).
-// 512 pairs of d = 3 (2.1e10 distances): see launch_scan_small_batch.
-template <int METRIC, int D, int PQ>
-__device__ __forceinline__ void small_item(int dtype, const void* __restrict__ A, const float* __restrict__ scA,
-                                           int64_t nA, const int64_t* __restrict__ qidx, int64_t T,
-                                           const void* __restrict__ B, const float* __restrict__ scB, int64_t b_begin,
-                                           int64_t b_end, int64_t l0, unsigned long long* __restrict__ best,
-                                           uint64_t* __restrict__ Bs) {
-  constexpr bool kL2 = METRIC == CH_L2;
-  constexpr int W = (kL2 ? D + 1 : D) + ((kL2 ? D + 1 : D) & 1);  // 64-bit words per row pair, even
-  const float kInf = __int_as_float(0x7F800000);
-  const int lane = threadIdx.x & 31;
-  const float u = 0x1p-24f;
-  auto load_q = [&](int p, float (&q)[D]) {
-    const int64_t l = l0 + 256 * p;
-    const int64_t a = l < T ? (qidx ? qidx[l] : l) : -1;
-#pragma unroll
-    for (int j = 0; j < D; ++j) q[j] = (a >= 0 && a < nA) ? elem_of(dtype, A, a, D, j, scA) : 0.0f;
-  };
-  uint64_t q2[PQ][D];
-  float b1[PQ], b2[PQ], b3[PQ];
-  int i1[PQ], i2[PQ];
-#pragma unroll
-  for (int p = 0; p < PQ; ++p) {
-    float q[D];
-    load_q(p, q);
-#pragma unroll
-    for (int j = 0; j < D; ++j) q2[p][j] = kL2 ? f2_pack(-2.0f * q[j], -2.0f * q[j]) : f2_pack(q[j], q[j]);
-    b1[p] = b2[p] = b3[p] = kInf;
-    i1[p] = i2[p] = -1;
-  }
-  for (int64_t s0 = b_begin; s0 < b_end; s0 += kSmallBT) {
-    const int rows = static_cast<int>(min(static_cast<int64_t>(kSmallBT), b_end - s0));
-    const int subs = (rows + kSmallSub - 1) / kSmallSub;
-    __syncthreads();
-    for (int f = threadIdx.x; f < subs * (kSmallSub / 2); f += 256) {
-      float v[2][D], n[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const bool ok = 2 * f + h < rows;
-        n[h] = ok ? 0.0f : kInf;
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          // past the end: +inf values for either metric
-          v[h][j] = ok ? elem_of(dtype, B, s0 + 2 * f + h, D, j, scB) : (kL2 ? 0.0f : kInf);
-          if (kL2 && ok) n[h] = __fmaf_rn(v[h][j], v[h][j], n[h]);
-        }
-        if (kL2) n[h] = __fmul_rd(n[h], 1.0f - 4 * D * u);
-      }
-      uint64_t* dst = Bs + size_t(f) * W;
-#pragma unroll
-      for (int j = 0; j < D; ++j) dst[j] = kL2 ? f2_pack(v[0][j], v[1][j]) : f2_pack(-v[0][j], -v[1][j]);
-      if (kL2) dst[D] = f2_pack(n[0], n[1]);
-    }
-    __syncthreads();
-    const int sub0 = static_cast<int>((s0 - b_begin) / kSmallSub);
-#pragma unroll 1
-    for (int sub = 0; sub < subs; ++sub) {
-      const ulonglong2* src = reinterpret_cast<const ulonglong2*>(Bs + size_t(sub) * (kSmallSub / 2) * W);
-      float m[PQ];
-#pragma unroll
-      for (int p = 0; p < PQ; ++p) m[p] = kInf;
-#pragma unroll 4
-      for (int r = 0; r < kSmallSub / 2; ++r) {
-        uint64_t w[W];
-#pragma unroll
-        for (int k = 0; k < W / 2; ++k) {
-          const ulonglong2 t = src[r * (W / 2) + k];
-          w[2 * k] = t.x;
-          w[2 * k + 1] = t.y;
-        }
-#pragma unroll
-        for (int p = 0; p < PQ; ++p) {
-          float2 v;
-          if constexpr (kL2) {
-            uint64_t acc = w[D];
-#pragma unroll
-            for (int j = 0; j < D; ++j) f2_fma(acc, q2[p][j], w[j]);
-            v = f2_unpack(acc);
-          } else {
-            float lo[D], hi[D];
-#pragma unroll
-            for (int j = 0; j < D; ++j) {
-              const float2 t = f2_unpack(f2_add(q2[p][j], w[j]));
-              lo[j] = fabsf(t.x);
-              hi[j] = fabsf(t.y);
-            }
-            v = make_float2(small_node<D, 0, 1>(lo), small_node<D, 0, 1>(hi));
-          }
-          m[p] = fmin3(m[p], v.x, v.y);
-        }
-      }
-#pragma unroll
-      for (int p = 0; p < PQ; ++p) {
-        const bool c1 = m[p] < b1[p];
-        if constexpr (kL2) {
-          b3[p] = fminf(b3[p], fmaxf(b2[p], m[p]));
-          i2[p] = c1 ? i1[p] : m[p] < b2[p] ? sub0 + sub : i2[p];
-          b2[p] = fminf(b2[p], fmaxf(b1[p], m[p]));
-        }
-        i1[p] = c1 ? sub0 + sub : i1[p];
-        b1[p] = fminf(b1[p], m[p]);
-      }
-    }
-  }
-  // the rows of sub-tile `sub`, one per lane (+inf past the end)
-  auto row_of = [&](int sub, float (&b)[D]) {
-    const int64_t r = b_begin + int64_t(sub) * kSmallSub + lane;
-    const bool ok = sub >= 0 && r < b_end;
-#pragma unroll
-    for (int j = 0; j < D; ++j) b[j] = ok ? elem_of(dtype, B, r, D, j, scB) : kInf;
-    return static_cast<uint32_t>(ok ? r : 0xFFFFFFFFll);
-  };
-#pragma unroll 1
-  for (int p = 0; p < PQ; ++p) {
-    if (l0 - threadIdx.x + 256 * p >= T) break;
-    // (p varies at run time: pick this group's trackers without indexing registers)
-    float t2 = kInf, t3 = kInf;
-    int e1 = -1, e2 = -1;
-#pragma unroll
-    for (int k = 0; k < PQ; ++k)
-      if (k == p) {
-        t2 = b2[k];
-        t3 = b3[k];
-        e1 = i1[k];
-        e2 = i2[k];
-      }
-    float q[D];
-    load_q(p, q);
-    uint32_t dmin = 0xFFFFFFFFu, imin = 0xFFFFFFFFu;  // this lane's sample: distance bits and index
-    float P = kInf;
-    // folds the warp's rows b (index r) into sample s
-    auto fold = [&](int s, const float (&qs)[D], const float (&b)[D], uint32_t r) {
-      const float v = small_canon<METRIC, D>(qs, b);
-      const uint32_t bits = r != 0xFFFFFFFFu ? __float_as_uint(kL2 ? __fsqrt_rn(v) : v) : 0xFFFFFFFFu;
-      const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, bits);
-      const uint32_t at = __reduce_min_sync(0xFFFFFFFFu, bits == least ? r : 0xFFFFFFFFu);
-      float least_p = 0.0f;
-      if constexpr (kL2) least_p = __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, r != 0xFFFFFFFFu ? __float_as_uint(v) : 0x7F800000u));
-      if (lane == s) {
-        if (least < dmin || (least == dmin && at < imin)) {
-          dmin = least;
-          imin = at;
-        }
-        P = fminf(P, least_p);
-      }
-    };
-#pragma unroll 1
-    for (int s = 0; s < 32; s += 4) {
-      float b[4][D];
-      uint32_t r[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) r[k] = row_of(__shfl_sync(0xFFFFFFFFu, e1, s + k), b[k]);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        float qs[D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) qs[j] = __shfl_sync(0xFFFFFFFFu, q[j], s + k);
-        fold(s + k, qs, b[k], r[k]);
-      }
-    }
-    if constexpr (kL2) {
-      float qn = 0.0f;
-#pragma unroll
-      for (int j = 0; j < D; ++j) qn = __fmaf_rn(q[j], q[j], qn);
-      const float thr = __fadd_ru(__fsub_ru(__fmul_ru(P, 1.0f + 0x1p-19f), __fmul_rd(qn, 1.0f - (2.125f * D + 2) * u)),
-                                  0x1p-100f);
-      const bool far = !(qn < 1e37f) || !(P < 1e37f) || t3 <= thr;  // the whole chunk
-      for (unsigned rest = __ballot_sync(0xFFFFFFFFu, !far && t2 <= thr); rest; rest &= rest - 1) {
-        const int s = __ffs(rest) - 1;
-        float qs[D], b[D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) qs[j] = __shfl_sync(0xFFFFFFFFu, q[j], s);
-        const uint32_t r = row_of(__shfl_sync(0xFFFFFFFFu, e2, s), b);
-        fold(s, qs, b, r);
-      }
-      for (unsigned rest = __ballot_sync(0xFFFFFFFFu, far); rest; rest &= rest - 1) {
-        const int s = __ffs(rest) - 1;
-        float qs[D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) qs[j] = __shfl_sync(0xFFFFFFFFu, q[j], s);
-        // a row per lane, folded once at the end
-        unsigned long long mine = ~0ull;
-#pragma unroll 4
-        for (int64_t r = b_begin + lane; r < b_end; r += 32) {
-          float b[D];
-#pragma unroll
-          for (int j = 0; j < D; ++j) b[j] = elem_of(dtype, B, r, D, j, scB);
-          const float v = __fsqrt_rn(small_canon<METRIC, D>(qs, b));
-          mine = min(mine, (static_cast<unsigned long long>(__float_as_uint(v)) << 32) | static_cast<uint32_t>(r));
-        }
-        const uint32_t least = __reduce_min_sync(0xFFFFFFFFu, static_cast<uint32_t>(mine >> 32));
-        const uint32_t at = __reduce_min_sync(0xFFFFFFFFu, (mine >> 32) == least ? static_cast<uint32_t>(mine) : 0xFFFFFFFFu);
-        if (lane == s) {
-          dmin = least;
-          imin = at;
-        }
-      }
-    }
-    const int64_t l = l0 + 256 * p;
-    // +inf and NaN (bits from 0x7F800000 on) are no minimum, as for the other scans
-    if (dmin >= 0x7F800000u) {
-      dmin = 0x7F800000u;
-      imin = 0xFFFFFFFFu;
-    }
-    if (l < T) atomicMin(&best[l], (static_cast<unsigned long long>(dmin) << 32) | imin);
-  }
-}
-
-// one pair: blockIdx.x = block of samples, blockIdx.y = chunk of B
-template <int METRIC, int D>
-__global__ void __launch_bounds__(256, 3) k_scan_small(int dtype, const void* __restrict__ A,
-                                                       const float* __restrict__ scA, const int64_t* __restrict__ qidx,
-                                                       int64_t T, int64_t nA, const void* __restrict__ B,
-                                                       const float* __restrict__ scB, int64_t nB, int64_t chunk_len,
-                                                       unsigned long long* best) {
-  pdl_entry();
-  __shared__ __align__(16) uint64_t Bs[kSmallBT / 2 * (D + 2)];
-  const int64_t b_begin = int64_t(blockIdx.y) * chunk_len;
-  small_item<METRIC, D, kSmallPQ>(dtype, A, scA, nA, qidx, T, B, scB, b_begin, min(nB, b_begin + chunk_len),
-                                  int64_t(blockIdx.x) * kSmallQ + threadIdx.x, best, Bs);
-}
-
-// The batched form: one persistent launch over items (pair, groups of 256 samples,
-// chunk of B) of many pairs of one storage type, metric and dimension, largest
-// first, each block taking the next one from a counter.
-template <int METRIC, int D>
-__global__ void __launch_bounds__(256, 2) k_scan_small_batch(int dtype, const SmallScanPair* __restrict__ pairs,
-                                                             const SmallScanItem* __restrict__ items, int64_t n_items,
-                                                             int64_t chunk_len, unsigned int* next) {
-  pdl_entry();
-  __shared__ __align__(16) uint64_t Bs[kSmallBT / 2 * (D + 2)];
-  __shared__ unsigned int s_w;
-  for (;;) {
-    __syncthreads();  // Bs and s_w are free again
-    if (threadIdx.x == 0) s_w = atomicAdd(next, 1u);
-    __syncthreads();
-    const int64_t w = s_w;
-    if (w >= n_items) return;
-    const SmallScanItem it = items[w];
-    const SmallScanPair pr = pairs[it.pair];
-    const int64_t l0 = int64_t(it.group) * 256 + threadIdx.x, b_end = min(pr.nB, it.b0 + chunk_len);
-    const auto run = [&](auto pq) {
-      small_item<METRIC, D, decltype(pq)::value>(dtype, pr.A, pr.scA, pr.nA, pr.qidx, pr.T, pr.B, pr.scB, it.b0, b_end,
-                                                 l0, pr.best, Bs);
-    };
-    switch (it.groups) {
-      case 1: case 2: run(std::integral_constant<int, 2>{}); break;
-      case 3: case 4: run(std::integral_constant<int, 4>{}); break;
-      case 5: run(std::integral_constant<int, 5>{}); break;
-      case 6: run(std::integral_constant<int, 6>{}); break;
-      case 7: run(std::integral_constant<int, 7>{}); break;
-      default: run(std::integral_constant<int, 8>{}); break;
-    }
-  }
-}
-
-// the lone small scan's minima to its outputs; best [segs][T], segment s holding the
-// rows from s * 2^31 on
-__global__ void k_scan_best_out(const unsigned long long* best, int segs, int64_t T, const int64_t* qidx, float* min_d,
-                                int64_t* argmin) {
-  pdl_entry();
-  const int64_t l = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (l >= T) return;
-  uint32_t bits = 0x7F800000u;
-  int64_t at = INT64_MAX;
-  for (int s = 0; s < segs; ++s) {
-    const unsigned long long v = best[s * T + l];
-    if (static_cast<uint32_t>(v >> 32) < bits) {
-      bits = static_cast<uint32_t>(v >> 32);
-      at = int64_t(s) * kSmallSegment + static_cast<int64_t>(v & 0xFFFFFFFFull);
-    }
-  }
-  const bool none = qidx && qidx[l] < 0;
-  min_d[l] = none ? 0.0f : __uint_as_float(bits);
-  if (argmin) argmin[l] = none ? -1 : at;
-}
-
 __global__ void k_scan_merge(const float* part_val, const int64_t* part_idx, int chunks, int64_t T,
                              const int64_t* qidx, float* min_d, int64_t* argmin) {
   pdl_entry();
@@ -721,12 +378,7 @@ static int scan_blocks_per_sm(int d, bool db) {
 }
 
 int scan_exact_chunks(int64_t T, int64_t nB, int d, int dtype, int sm_count) {
-  if (d <= kSmallMaxD) {  // k_scan_small: about 4 blocks per SM, chunks of >= 256 points
-    const int64_t qblocks = ceil_div(std::max<int64_t>(T, 1), kSmallQ);
-    int64_t chunks = ceil_div(int64_t(sm_count) * 4, qblocks);
-    chunks = std::min<int64_t>(chunks, ceil_div(nB, 256));
-    return static_cast<int>(std::max<int64_t>(chunks, 1));
-  }
+  if (d <= kScanSmallMaxD) return scan_small_chunks(T, nB, sm_count);
   // B is cut into equal chunks, one block per (sample tile, chunk).  The count
   // minimises (waves of resident blocks) x (B tiles per block), the kernel's time
   // when every wave runs at the same rate; ties go to fewer chunks (less merging).
@@ -796,40 +448,9 @@ static void scan_shape(const ch_set* A, const int64_t* qidx, int64_t T, const ch
     scan_launch<DT, METRIC, 16, 16, 1, 1>(A, qidx, T, B, part, s, list);
 }
 
-template <int METRIC>
-static void scan_small(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, ScanPart part,
-                       cudaStream_t s) {
-  const int segs = scan_small_segments(B->n);
-  CHX_CUDA(cudaMemsetAsync(part.best, 0xFF, size_t(segs) * T * sizeof(unsigned long long), s));
-  for (int g = 0; g < segs; ++g) {
-    const int64_t n0 = int64_t(g) * kSmallSegment, n = std::min(kSmallSegment, B->n - n0);
-    const char* base = static_cast<const char*>(B->data) + size_t(n0) * A->d * elem_size(B->dtype);
-    const float* sc = B->scales ? B->scales + n0 : nullptr;
-    const int64_t chunk_len = ceil_div(n, part.chunks);
-    const dim3 grid(static_cast<unsigned>(ceil_div(T, kSmallQ)), static_cast<unsigned>(part.chunks));
-    auto go = [&](auto kern) {
-      launch_k(kern, grid, 256, 0, s, A->dtype, A->data, A->scales, qidx, T, A->n, base, sc, n, chunk_len,
-               part.best + size_t(g) * T);
-    };
-    switch (A->d) {
-      case 1: go(k_scan_small<METRIC, 1>); break;
-      case 2: go(k_scan_small<METRIC, 2>); break;
-      case 3: go(k_scan_small<METRIC, 3>); break;
-      default: go(k_scan_small<METRIC, 4>); break;
-    }
-  }
-}
-
 template <int DT>
 static void scan_metric(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, ScanPart part,
                         cudaStream_t s) {
-  if (A->d <= kSmallMaxD) {
-    if (metric == CH_L1)
-      scan_small<CH_L1>(A, qidx, T, B, part, s);
-    else
-      scan_small<CH_L2>(A, qidx, T, B, part, s);
-    return;
-  }
   if (metric == CH_L1)
     scan_shape<DT, CH_L1>(A, qidx, T, B, part, s);
   else
@@ -840,6 +461,7 @@ void launch_scan_exact(const ch_set* A, const int64_t* qidx, int64_t T, const ch
                        int sm_count, cudaStream_t s) {
   (void)sm_count;
   if (T == 0) return;
+  if (A->d <= kScanSmallMaxD) return launch_scan_small(A, qidx, T, B, metric, part, s);
   CHX_CHECK(scan_fits(A->d), CH_ENOTSUP, "dimension too large for the exact scan");
   switch (A->dtype) {
     case CH_F32: scan_metric<CH_F32>(A, qidx, T, B, metric, part, s); break;
@@ -849,17 +471,10 @@ void launch_scan_exact(const ch_set* A, const int64_t* qidx, int64_t T, const ch
   launch_check("scan_exact");
 }
 
-int scan_small_segments(int64_t nB) { return static_cast<int>(std::max<int64_t>(1, ceil_div(nB, kSmallSegment))); }
-
 void launch_scan_merge(ScanPart part, int64_t T, int64_t nB, const int64_t* qidx, float* min_d, int64_t* argmin,
                        cudaStream_t s) {
   if (T == 0) return;
-  if (part.best) {
-    launch_k(k_scan_best_out, static_cast<int>(ceil_div(T, 256)), 256, 0, s, part.best, scan_small_segments(nB), T, qidx,
-             min_d, argmin);
-    launch_check("scan_best_out");
-    return;
-  }
+  if (part.best) return launch_scan_small_out(part, T, nB, qidx, min_d, argmin, s);
   launch_k(k_scan_merge, static_cast<int>(ceil_div(T, 256)), 256, 0, s, part.val, part.idx, part.chunks, T, qidx, min_d,
                                                                   argmin);
   launch_check("scan_merge");
@@ -881,35 +496,6 @@ void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
   launch_k(k_scan_list_out, static_cast<int>(std::min<int64_t>(ceil_div(T, 256), sm_count)), 256, 0, s, sl, min_d,
            argmin);
   launch_check("scan_list_out");
-}
-
-int small_scan_max_groups() { return kBatchPQ; }
-
-template <int METRIC>
-static void small_batch_d(const SmallScanPair* pairs, const SmallScanItem* items, int64_t n, int64_t chunk_len,
-                          int dtype, int d, int grid, unsigned int* next, cudaStream_t s) {
-  auto go = [&](auto kern) { launch_k(kern, grid, 256, 0, s, dtype, pairs, items, n, chunk_len, next); };
-  switch (d) {
-    case 1: go(k_scan_small_batch<METRIC, 1>); break;
-    case 2: go(k_scan_small_batch<METRIC, 2>); break;
-    case 3: go(k_scan_small_batch<METRIC, 3>); break;
-    default: go(k_scan_small_batch<METRIC, 4>); break;
-  }
-}
-
-void launch_scan_small_batch(const SmallScanPair* pairs, const SmallScanItem* items, int64_t n_items,
-                             int64_t chunk_len, int dtype, int metric, int d, unsigned int* next, int sm_count,
-                             cudaStream_t s) {
-  if (n_items == 0) return;
-  CHX_CHECK(d >= 1 && d <= kSmallMaxD, CH_EINVAL, "batched small scan: d must be in 1..4");
-  CHX_CUDA(cudaMemsetAsync(next, 0, sizeof(unsigned int), s));
-  // a persistent grid of two resident blocks per SM
-  const int grid = static_cast<int>(std::min<int64_t>(n_items, int64_t(sm_count) * 2));
-  if (metric == CH_L1)
-    small_batch_d<CH_L1>(pairs, items, n_items, chunk_len, dtype, d, grid, next, s);
-  else
-    small_batch_d<CH_L2>(pairs, items, n_items, chunk_len, dtype, d, grid, next, s);
-  launch_check("scan_small_batch");
 }
 
 }  // namespace chx
