@@ -598,7 +598,7 @@ struct CertArgs {
   double p_scale, q_scale;  // a column is evaluated when L <= P p_scale - |q|^2 q_scale + 2^-100
   int64_t limit;            // most columns evaluated per sample
   int32_t* list;            // samples left to k_scan_exact's list form
-  uint32_t* ctl;            // [0] their number, [1] set when a screen gave up
+  uint32_t* ctl;            // [0] their number, [1] set when a screen gave up, [2] the list form's ended blocks
   unsigned long long* best; // [T of the call] the list form's minima, set to all ones with each listing
 };
 void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, int metric, const CertArgs& c, float* min_d,
@@ -608,7 +608,7 @@ void launch_certify(const ch_set* A, const int64_t* qidx, const ch_set* B, int m
 bool scan_list_fits(int64_t T, int d);
 // the exact scan of the ctl[0] listed samples (at most T), written to their places
 void launch_scan_list(const ch_set* A, const int64_t* qidx, int64_t T, const ch_set* B, int metric, const int32_t* list,
-                      const uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,
+                      uint32_t* ctl, unsigned long long* best, float* min_d, int64_t* argmin, int sm_count,
                       cudaStream_t s);
 
 // result block copied to the host at the end of a synchronising call

@@ -286,7 +286,7 @@ void launch_exact_chain(const ch_set* A, const int64_t* qidx, int64_t T, const c
   w += al(size_t(T) * 4);
   c.best = reinterpret_cast<unsigned long long*>(w);
   w += al(size_t(T) * 8);
-  CHX_CUDA(cudaMemsetAsync(c.ctl, 0, 8, s));
+  CHX_CUDA(cudaMemsetAsync(c.ctl, 0, 12, s));
   c.d = d;
   c.nB = B->n;
   c.p_scale = 1.0 + 0x1p-20 + 2.0 * (d + d / 32 + 12) * 0x1p-24;

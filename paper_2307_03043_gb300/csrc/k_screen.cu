@@ -774,7 +774,7 @@ void launch_exact_tc(const ch_set* A, const int64_t* qidx, int64_t T, const ch_s
   const int64_t Ts = std::min(T, kCertSlice);
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   char* w = static_cast<char*>(work);
-  uint32_t* ctl = reinterpret_cast<uint32_t*>(w);  // [0] listed samples, [1] a screen gave up
+  uint32_t* ctl = reinterpret_cast<uint32_t*>(w);  // see CertArgs
   w += 256;
   int32_t* list = reinterpret_cast<int32_t*>(w);
   w += al(size_t(T) * 4);
@@ -782,7 +782,7 @@ void launch_exact_tc(const ch_set* A, const int64_t* qidx, int64_t T, const ch_s
   w += al(size_t(T) * 8);
   uint8_t* Q = reinterpret_cast<uint8_t*>(w);
   w += al(size_t(Ts) * row_bytes);
-  CHX_CUDA(cudaMemsetAsync(ctl, 0, 8, s));
+  CHX_CUDA(cudaMemsetAsync(ctl, 0, 12, s));
 
   const double c_in = screen == CH_SCREEN_TF32 ? 0x1p-9 * (1.0 + 0x1p-10) : 0.0;
   const double a_half = (c_in + 4.0 * d * 0x1p-23) + 0x1p-23;

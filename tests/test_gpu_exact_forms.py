@@ -1,0 +1,125 @@
+"""The exact scan's forms for d > 4 where they meet ties: FP8 rows with scales in the
+chained form, samples left to the list form in each of its tile shapes, queries repeated
+in B, and sets off the origin.  Bit for bit the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_03043_gb300 import binding as ch
+from paper_2307_03043_gb300 import workloads
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DTYPES = {"f32": ch.CH_F32, "bf16": ch.CH_BF16, "fp8": ch.CH_FP8E4M3}
+METRICS = {"l1": ch.CH_L1, "l2": ch.CH_L2}
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2307_03043_gb300 import build
+    build.build()
+    c = ch.ch_ctx_create(0, torch.cuda.current_stream())
+    yield c
+    ch.ch_ctx_destroy(c)
+
+
+def _stored(X, dtype):
+    """(device rows, device scales or None, the values the library sees)."""
+    if dtype == ch.CH_BF16:
+        h = workloads.to_bf16_bits(X)
+        return torch.from_numpy(h.view(np.int16)).cuda(), None, workloads.bf16_bits_to_f32(h)
+    if dtype == ch.CH_FP8E4M3:
+        codes, scales = workloads.to_fp8_e4m3(X)
+        return torch.from_numpy(codes).cuda(), torch.from_numpy(scales).cuda(), workloads.fp8_dequant(codes, scales)
+    return torch.from_numpy(X).cuda(), None, X
+
+
+def _make(ctx, X, dtype):
+    rows, scales, seen = _stored(np.ascontiguousarray(X, dtype=np.float32), dtype)
+    return ch.ch_set_create(ctx, rows, 2 if scales is None else 1, *X.shape, dtype, scales), (rows, scales), seen
+
+
+def _check(ctx, A, B, idx, dtype, metric):
+    sA, keepA, A = _make(ctx, A, dtype)
+    sB, keepB, B = _make(ctx, B, dtype)
+    T = idx.size
+    m = torch.full((T,), -1.0, device="cuda")
+    am = torch.full((T,), -7, dtype=torch.int64, device="cuda")
+    ch.ch_sampled_nn(ctx, sA, torch.from_numpy(idx).cuda(), T, sB, metric, ch.CH_SCREEN_EXACT, 8, m, am)
+    mo, amo = oracle.scan(A, idx, B, metric)
+    assert np.array_equal(m.cpu().numpy().view(np.uint32), mo.view(np.uint32))
+    assert np.array_equal(am.cpu().numpy(), amo)
+    for s in (sA, sB):
+        ch.ch_set_destroy(s)
+
+
+def _draw(n, T, seed=1):
+    idx = np.random.default_rng(seed).integers(0, n, T).astype(np.int64)
+    idx[3::29] = -1
+    return idx
+
+
+# rows of a lane each, of a lane group each (512 bytes and more), and of any length
+@pytest.mark.parametrize("metric", list(METRICS))
+@pytest.mark.parametrize("nB,d,T", [(8501, 64, 1000), (9601, 97, 600), (1901, 512, 600), (1050, 1040, 530)])
+@pytest.mark.parametrize("ties", [False, True], ids=["plain", "ties"])
+def test_fp8_chained(ctx, metric, nB, d, T, ties):
+    A, B = workloads.gaussian_mixture(500, nB, d, nB + d, clusters=5)
+    if ties:
+        B[nB // 2:] = B[:nB - nB // 2]
+        B[5::7] = B[5]
+        A[::9] = B[5] + np.float32(0.5)
+    _check(ctx, A, B, _draw(500, T), ch.CH_FP8E4M3, METRICS[metric])
+
+
+# every tile shape of the list form, reached with all samples (one row repeated through B)
+# and with some of them (those nearest to a row that half of B repeats)
+@pytest.mark.parametrize("metric", list(METRICS))
+@pytest.mark.parametrize("dtype", list(DTYPES))
+@pytest.mark.parametrize("nB,d,T", [(16500, 8, 4200), (20001, 33, 900), (8501, 64, 1100), (7001, 97, 900), (8001, 128, 530),
+                                    (5003, 200, 600), (3501, 300, 600), (1050, 1000, 600)])
+@pytest.mark.parametrize("listed", ["all", "some"])
+def test_list_form(ctx, metric, dtype, nB, d, T, listed):
+    A, B = workloads.gaussian_mixture(600, nB, d, nB + d, clusters=5)
+    if listed == "all":
+        B[:] = B[3]
+    else:
+        B[1::2] = B[1]
+        A[::11] = B[1] + np.float32(0.25)
+    _check(ctx, A, B, _draw(600, T), DTYPES[dtype], METRICS[metric])
+
+
+@pytest.mark.parametrize("metric", list(METRICS))
+@pytest.mark.parametrize("dtype", list(DTYPES))
+@pytest.mark.parametrize("d,cells", [(8, 2), (8, 4), (16, 2), (64, 2)])
+def test_queries_repeated_in_b(ctx, metric, dtype, d, cells):
+    g = np.random.default_rng(d * cells)
+    A = g.integers(0, cells, (700, d)).astype(np.float32)
+    B = g.integers(0, cells, (30011, d)).astype(np.float32)
+    B[20000:20700] = A
+    _check(ctx, A, B, _draw(700, 2300), DTYPES[dtype], METRICS[metric])
+
+
+@pytest.mark.parametrize("d", [8, 16, 128])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("brute", [False, True], ids=["drawn", "in_order"])
+def test_far_off_sets(ctx, d, dtype, brute):
+    """l2 sets 1000 off the origin: the bound excludes nothing, and every sample (in A's
+    order, more than one slice of them) goes to the list form."""
+    nA = 17000 if brute else 900
+    A, B = workloads.gaussian_mixture(nA, 3001, d, 4 + d, clusters=6)
+    A, B = A + np.float32(1000), B + np.float32(1000)
+    if not brute:
+        _check(ctx, A, B, _draw(nA, 1500), DTYPES[dtype], ch.CH_L2)
+        return
+    sA, keepA, A = _make(ctx, A, DTYPES[dtype])
+    sB, keepB, B = _make(ctx, B, DTYPES[dtype])
+    mins = torch.zeros(nA, device="cuda")
+    v = ch.ch_exact(ctx, sA, sB, ch.CH_L2, 0, mins)
+    vo, mo = oracle.exact_canonical(A, B, ch.CH_L2)
+    assert np.array_equal(mins.cpu().numpy(), mo) and abs(v / vo - 1) < 1e-12
+    for s in (sA, sB):
+        ch.ch_set_destroy(s)
