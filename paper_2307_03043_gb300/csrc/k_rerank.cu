@@ -283,13 +283,16 @@ namespace {
 // is evaluated: the four columns of each class entry at or below the threshold and,
 // where a class's second-smallest tile minimum is at or below it too, all of the
 // class's columns in the chunk.  The entries collect in a queue, eight at a time
-// give a column to every lane, and a lane computes its column's distance alone (no
-// shuffles, 32 rows in flight); the threshold tightens after each such batch.  A
-// sample with more than c.limit columns, with values outside the bound's range, or
-// whose screen gave up is listed instead.
+// give a column to every lane, and the warp computes the 32 distances in the form its
+// rows allow (FORM below); the threshold tightens after each such batch.  A point
+// at distance 0 leaves only smaller indices to look at: however often a query is
+// repeated in B, its first copy answers it.  A sample with more than c.limit columns,
+// with values outside the bound's range, or whose screen gave up is listed instead.
 constexpr int kCertQueue = 8 + 32;  // a batch and the entries one part can add
 
-// FORM: how a batch's distances are formed.
+// FORM: how a batch's distances are formed.  Rows of a multiple of 16 bytes on aligned
+// bases: a row per lane (lane_dist) or, from kWideRow bytes on, per lane group
+// (group_dist); any others: CF_ROWS.
 enum : int { CF_LANE = 0, CF_GROUP = 1, CF_ROWS = 2 };
 
 // CF_ROWS, for rows of any length: four rows at a time, lane r summing coordinates
@@ -434,14 +437,27 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
     give_up();
     return;
   }
+  // a point at distance 0 (its index): none from it on matters
+  const uint32_t stop = bestP == 0.0f ? __reduce_min_sync(0xFFFFFFFFu, best == 0.0f ? bidx : 0xFFFFFFFFu) : 0xFFFFFFFFu;
   // columns to evaluate under this threshold
   const int64_t tiles = c.chunk_len / c.tile;
   int64_t cols = 0;
+  if (stop == 0xFFFFFFFFu) {
 #pragma unroll 4
-  for (int p = 0; p < c.parts; ++p) {
-    const bool e = __ldg(&c.part_s[p * stride + at]) <= thr;
-    const bool all = __ldg(&c.part_2[p * stride + at]) <= thr;
-    cols += 4 * __popc(__ballot_sync(0xFFFFFFFFu, e && !all)) + 4 * tiles * __popc(__ballot_sync(0xFFFFFFFFu, all));
+    for (int p = 0; p < c.parts; ++p) {
+      const bool e = __ldg(&c.part_s[p * stride + at]) <= thr;
+      const bool all = __ldg(&c.part_2[p * stride + at]) <= thr;
+      cols += 4 * __popc(__ballot_sync(0xFFFFFFFFu, e && !all)) + 4 * tiles * __popc(__ballot_sync(0xFFFFFFFFu, all));
+    }
+  } else {  // entries and tiles before it
+    for (int p = 0; p < c.parts; ++p) {
+      const int64_t c0 = int64_t(p / c.slices) * c.chunk_len + (p % c.slices) * c.slice_cols + lane * c.class_cols;
+      const int64_t n = (int64_t(stop) - c0 + c.tile - 1) / c.tile;
+      const int64_t mine = __ldg(&c.part_2[p * stride + at]) <= thr ? max(int64_t(0), min(tiles, n))
+                           : __ldg(&c.part_s[p * stride + at]) <= thr &&
+                                 static_cast<uint32_t>(__ldg(&c.part_i[p * stride + at])) < stop;
+      cols += 4 * int64_t(__reduce_add_sync(0xFFFFFFFFu, static_cast<uint32_t>(mine)));
+    }
   }
   if (cols > c.limit) {
     give_up();
@@ -465,7 +481,7 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
     const float s2 = __ldg(&c.part_2[p * stride + at]);
     const int32_t i = __ldg(&c.part_i[p * stride + at]);
     const unsigned all = __ballot_sync(0xFFFFFFFFu, s2 <= thr);
-    const bool mine = s1 <= thr && i >= 0 && i != mi && !(all >> lane & 1u);
+    const bool mine = s1 <= thr && i != mi && static_cast<uint32_t>(i) < stop && !(all >> lane & 1u);
     const unsigned one = __ballot_sync(0xFFFFFFFFu, mine);
     if (mine) queue[n + __popc(one & ((1u << lane) - 1u))] = i;
     n += __popc(one);
@@ -473,7 +489,7 @@ __global__ void __launch_bounds__(32 * kRerankWarps, 2) k_certify(const void* A,
     for (unsigned rest = all; rest; rest &= rest - 1) {
       const int64_t c0 =
           int64_t(p / c.slices) * c.chunk_len + (p % c.slices) * c.slice_cols + (__ffs(rest) - 1) * c.class_cols;
-      const int64_t end = min(c.nB, (int64_t(p / c.slices) + 1) * c.chunk_len);
+      const int64_t end = min(min(c.nB, int64_t(stop)), (int64_t(p / c.slices) + 1) * c.chunk_len);
       for (int64_t b = c0; b < end; b += 32 * int64_t(c.tile)) {  // 32 tiles of the class at a time
         const int64_t mb = b + int64_t(lane) * c.tile;
         if (mb < end) queue[n + lane] = static_cast<int32_t>(mb);

@@ -103,6 +103,35 @@ def test_queries_repeated_in_b(ctx, metric, dtype, d, cells):
     _check(ctx, A, B, _draw(700, 2300), DTYPES[dtype], METRICS[metric])
 
 
+def _best_ms(ctx, A, B, T, metric):
+    sA, keepA, _ = _make(ctx, A, ch.CH_F32)
+    sB, keepB, _ = _make(ctx, B, ch.CH_F32)
+    idx = torch.from_numpy(np.random.default_rng(1).integers(0, A.shape[0], T).astype(np.int64)).cuda()
+    m = torch.empty(T, device="cuda")
+    best = float("inf")
+    for _ in range(10):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        ch.ch_sampled_nn(ctx, sA, idx, T, sB, metric, ch.CH_SCREEN_EXACT, 8, m)
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1))
+    for s in (sA, sB):
+        ch.ch_set_destroy(s)
+    return best
+
+
+@pytest.mark.parametrize("metric", list(METRICS))
+def test_repeated_queries_cost_little(ctx, metric):
+    """Corners of the cube of d = 8, each some 400 times in B and in A: k_certify settles
+    them.  (Listed instead, they took 3.3 times the mixture's time in l1, 8 times in l2; 2
+    leaves room for noise.)"""
+    g = np.random.default_rng(3)
+    corners = [g.integers(0, 2, (n, 8)).astype(np.float32) for n in (20000, 100000)]
+    mixture = workloads.gaussian_mixture(20000, 100000, 8, 4)
+    assert _best_ms(ctx, *corners, 4606, METRICS[metric]) < 2 * _best_ms(ctx, *mixture, 4606, METRICS[metric])
+
+
 @pytest.mark.parametrize("d", [8, 16, 128])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("brute", [False, True], ids=["drawn", "in_order"])
