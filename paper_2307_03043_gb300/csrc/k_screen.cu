@@ -732,24 +732,38 @@ void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
 // column whose canonical distance ties with or beats a known P has
 //   L(b) <= P (1 + 2^-20 + 2 g) - |q|^2 (1 - a/2 - (d/32 + 8) 2^-23) + 2^-100
 // (the last factor covers |q|^2's own rounding, 2^-100 every underflow).  k_certify evaluates
-// every column that meets this; samples with too many of them, or out of the
-// bound's range, go to k_scan_exact's list form.
+// every column that meets this; samples with too many of them, or out of the bound's
+// range, go to k_scan_exact's list form.  Sets far from the origin pay for nothing: where
+// a |b|^2 (|b|^2 / 256 for binary32 rows) passes the nearest squared distances, every
+// sample is listed, and the call takes the plain scan's time and the screen's (T = 4606 x
+// 100k of unit clusters, 30 off the origin: d = 8 0.88 -> 1.03 ms, d = 128 5.4 -> 5.9 ms;
+// 0.14 and 0.28 ms at the origin).  A kernel that looked at 16 samples x 512 rows first
+// and skipped the screen brought those to 0.93 and 5.75 ms, but cost every other call 9 to
+// 20 us (6 to 17 % of those above), so it was left out.
 
 // samples per launch of the certified scan: bounds its scratch (about 100 MB of
 // candidates) whatever |A| is; 128 sample tiles still fill the SMs
 constexpr int64_t kCertSlice = 16384;
 
 // From 128 samples (a whole tile) and 2^20 pairs on, 2^23 below 512 samples, whose few
-// tiles leave SMs idle (k_scan_exact / certified: 1024 x 1024, d = 16 31 / 27 us; 512 x
-// 2048, d = 128 34.5 / 32.5 us; 2048 x 2048, d = 32 41 / 34 us; 256 x 4096, d = 64 22 / 39
-// us; 20k x 30k, d = 128 7.26 ms / 0.45 ms).
+// tiles leave SMs idle; where the plain scan's tiles are cheap, from so many (sample,
+// point, coordinate) terms on: d <= 16 (256-row stages) 92 M, 32 < d <= 64 230 M.  On the
+// device, plain / certified, uniform points: d = 8 1000 x 4000 28 / 43 us, 3000 x 4000
+// (96 M) 41 / 43, 3000 x 6000 55 / 45; d = 16 3000 x 1500 34 / 41, 3000 x 2000 (96 M)
+// 41 / 35; d = 24 1000 x 2000 37 / 32; d = 32 1000 x 1500 34 / 30; d = 40 3000 x 1500
+// (180 M) 39 / 43, 3000 x 2000 (240 M) 49 / 38; d = 64 1000 x 2000 28 / 34, 3000 x 1500
+// (288 M) 49 / 43; d = 96 1000 x 1500 39 / 32; 256 samples x 4096, d = 64 22 / 39; 20k x
+// 30k, d = 128 7.24 / 0.44 ms.
 bool exact_tc_supported(const ch_set* A, const ch_set* B, int64_t T) {
   if (A->dtype != B->dtype || (A->dtype != CH_F32 && A->dtype != CH_BF16)) return false;
   const int64_t row = int64_t(A->d) * int64_t(elem_size(A->dtype));
   if (A->d <= 4 || row % 16 != 0 || row > 16384) return false;
   if ((reinterpret_cast<uintptr_t>(A->data) & 15) || (reinterpret_cast<uintptr_t>(B->data) & 15)) return false;
-  return T >= kBM && B->n >= kBN && B->n < (int64_t(1) << 31) && T * B->n >= int64_t(T >= 512 ? 1 << 20 : 1 << 23) &&
-         scan_list_fits(T, A->d);
+  if (T < kBM || B->n < kBN || B->n >= (int64_t(1) << 31) || !scan_list_fits(T, A->d)) return false;
+  const double pairs = double(T) * double(B->n);
+  if (T < 512) return pairs >= double(1 << 23);
+  const double terms = A->d <= 16 ? 92e6 : A->d > 32 && A->d <= 64 ? 230e6 : 0.0;
+  return pairs >= double(1 << 20) && pairs * A->d >= terms;
 }
 
 static int cert_screen(int dtype) { return dtype == CH_F32 ? CH_SCREEN_TF32 : CH_SCREEN_BF16; }

@@ -142,11 +142,32 @@ def test_far_off_sets(ctx, d, dtype, brute):
     A, B = workloads.gaussian_mixture(nA, 3001, d, 4 + d, clusters=6)
     A, B = A + np.float32(1000), B + np.float32(1000)
     if not brute:
-        _check(ctx, A, B, _draw(nA, 1500), DTYPES[dtype], ch.CH_L2)
+        _check(ctx, A, B, _draw(nA, 4200), DTYPES[dtype], ch.CH_L2)
         return
     sA, keepA, A = _make(ctx, A, DTYPES[dtype])
     sB, keepB, B = _make(ctx, B, DTYPES[dtype])
     mins = torch.zeros(nA, device="cuda")
+    v = ch.ch_exact(ctx, sA, sB, ch.CH_L2, 0, mins)
+    vo, mo = oracle.exact_canonical(A, B, ch.CH_L2)
+    assert np.array_equal(mins.cpu().numpy(), mo) and abs(v / vo - 1) < 1e-12
+    for s in (sA, sB):
+        ch.ch_set_destroy(s)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("nB,d,T", [(257, 8, 46000), (1000, 16, 6000), (5003, 8, 2400), (4099, 40, 1500),
+                                    (2049, 64, 1800)])
+def test_certified_edges_of_its_rule(ctx, dtype, nB, d, T):
+    """The certified form's tile, slice and row edges at the smallest calls that take it."""
+    A, B = workloads.gaussian_mixture(900, nB, d, nB + d, clusters=5)
+    _check(ctx, A, B, _draw(900, T), DTYPES[dtype], ch.CH_L2)
+
+
+def test_certified_brute_force_over_slices_of_small_rows(ctx):
+    A, B = workloads.uniform(17000, 601, 12, 5)
+    sA, keepA, _ = _make(ctx, A, ch.CH_F32)
+    sB, keepB, _ = _make(ctx, B, ch.CH_F32)
+    mins = torch.zeros(17000, device="cuda")
     v = ch.ch_exact(ctx, sA, sB, ch.CH_L2, 0, mins)
     vo, mo = oracle.exact_canonical(A, B, ch.CH_L2)
     assert np.array_equal(mins.cpu().numpy(), mo) and abs(v / vo - 1) < 1e-12

@@ -49,8 +49,10 @@ def test_rules_at_their_other_edges(rules):
     cases = {
         (1, 1): [_case(), _case(d=384, dtype=ch.CH_BF16)],
         (0, 1): [_case(d=33), _case(d=64, alignB=4), _case(d=64, alignA=8), _case(d=64, dtype=ch.CH_FP8E4M3)],
-        (1, 0): [_case(T=256, nB=40000, d=16), _case(T=1024, nB=1024, d=16)],
-        (0, 0): [_case(d=4), _case(nB=2 ** 31), _case(T=100), _case(T=512, nB=200, d=16)],
+        (1, 0): [_case(T=256, nB=40000, d=16), _case(T=1024, nB=1024, d=32), _case(T=3000, nB=2000, d=16),
+                 _case(T=3000, nB=4000, d=8), _case(T=3000, nB=2000, d=40)],
+        (0, 0): [_case(d=4), _case(nB=2 ** 31), _case(T=100), _case(T=512, nB=200, d=16),
+                 _case(T=1024, nB=1024, d=16), _case(T=3000, nB=3000, d=8), _case(T=1000, nB=2000, d=64)],
     }
     for want, cs in cases.items():
         assert rules(*cs) == [want] * len(cs), want
