@@ -54,13 +54,16 @@ typedef enum { CH_L1 = 1, CH_L2 = 2 } ch_metric;
 typedef enum { CH_F32 = 0, CH_BF16 = 1, CH_FP8E4M3 = 2 } ch_dtype;
 
 /* How the sampled l2 scan finds min_b d(q, b):
- *  EXACT  canonical binary32 distance to every b (CUDA cores);
+ *  EXACT  the minimum of the canonical binary32 distance over every b, bit for bit: by
+ *         the canonical distances of all pairs (CUDA cores), or by a tensor-core screen
+ *         (rows the screen reads) or chained binary32 sums (other rows) with an error
+ *         bound, and the canonical distance of every b that the bound leaves;
  *  TF32/BF16/FP8  tensor-core screen of |b|^2 - 2 q.b; per sample it keeps
  *         screened entries (4 columns of B each, scored by their best column),
  *         takes the rerank_k best entries and evaluates the canonical
  *         distance on all their columns;
  *  AUTO   TF32 for F32 sets, BF16 for BF16 sets, FP8 for FP8 sets.
- * l1 always uses the exact CUDA-core scan. */
+ * l1 always uses the exact scan, on CUDA cores. */
 typedef enum {
     CH_SCREEN_AUTO = 0,
     CH_SCREEN_EXACT = 1,
@@ -72,7 +75,8 @@ typedef enum {
 /* CrudeNN grouping of equal bucket keys (Fig. 2, step 3):
  *  HASH  open-addressing table of B's buckets per scale, probed by each a in
  *        increasing scale order (the structure Fig. 2 describes);
- *  SORT  device radix sort of (scale, key) with segmented minima.
+ *  SORT  device radix sort of B's keys, a segment per scale; each a finds its buckets
+ *        in the sorted segments by binary search.
  * Both give bit-identical b(a). */
 typedef enum { CH_GROUP_HASH = 0, CH_GROUP_SORT = 1 } ch_group;
 
@@ -162,8 +166,10 @@ int64_t ch_ctx_workspace_bytes(const ch_ctx* ctx);
  * l2 scan), in SM clock cycles; 0 (the default) means about 2 s.  A wait that
  * runs out stops the kernel's work; the kernel still waits, within the default
  * bound, for every copy and tensor-core operation it issued before it frees its
- * memory, and the call returns CH_ETIMEOUT with the context still usable.  A
- * small budget turns a stalled pipeline into that error quickly.  Applies to the
+ * memory, and the call returns CH_ETIMEOUT with the context still usable.  (The
+ * exact scan does not need its screen: where that gives up, its samples are scanned
+ * on CUDA cores and the call succeeds.)  A small budget turns a stalled pipeline
+ * into that error quickly.  Applies to the
  * context's later calls (and to the lanes of its batched calls).  CH_EINVAL for
  * a negative value or a NULL context. */
 ch_status ch_ctx_set_wait_cycles(ch_ctx* ctx, int64_t cycles);
@@ -294,7 +300,9 @@ ch_status ch_estimate_batch(ch_ctx* ctx, int64_t count, const ch_set* const* A, 
  * CH(A, B) + CH(B, A) (Section 1's symmetric Chamfer distance) as two one-sided
  * estimates under the same parameters, except that the (B, A) draws use the key
  * sample_seed ^ 0x9E3779B97F4A7C15; T = 0 gives both directions the default T of
- * max(|A|, |B|).  The two directions run concurrently (as a batch of two).
+ * max(|A|, |B|).  The directions share both sets' passes and follow one another on the
+ * context's stream; the variants without shared passes (k x W, SimHash, sort grouping,
+ * uniform sampling) run as a batch of two.
  * eta: host, the sum; eta_ab / eta_ba: host, each direction, or NULL.  Errors as
  * ch_estimate (the first failing direction's status). */
 ch_status ch_estimate_sym(ch_ctx* ctx, const ch_set* A, const ch_set* B, const ch_est_params* p, double* eta,

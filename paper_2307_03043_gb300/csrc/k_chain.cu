@@ -259,7 +259,10 @@ void chain_launch(const ch_set* A, const int64_t* qidx, int64_t l0, int64_t n, c
 // k_scan_exact is one launch and fills the SMs with less (l1, k_scan_exact / chained:
 // T = 2000 x 4000, d = 64, 2^28.9: 63.6 / 63.7 us; T = 128 x 20k, d = 64: 45 / 64 us;
 // T = 64 x 50k, d = 128: 82 / 111 us; T = 4.6k x 100k, d = 64: 2.90 / 2.0 ms; T = 3k x
-// 20k, d = 300 bf16: 2.47 / 1.46 ms).
+// 20k, d = 300 bf16: 2.47 / 1.46 ms).  A sample with hundreds of rows at one distance
+// other than 0 is listed and pays for both (T = 4.6k x 100k, every row of B the same: d =
+// 8 0.73 / 1.29 ms, d = 64 2.90 / 5.15 ms); small whole coordinates do not come to that
+// (in [0, 4) or [0, 16): 0.53 ms at d = 8), nor does B a hundred times over (0.54 ms).
 bool exact_chain_pays(const ch_set* A, const ch_set* B, int64_t T) {
   return A->d > 4 && A->dtype == B->dtype && T >= 512 && B->n < (int64_t(1) << 31) && scan_list_fits(T, A->d) &&
          double(T) * double(B->n) * A->d >= double(1 << 29);

@@ -545,8 +545,8 @@ __global__ void __launch_bounds__(kBatchThreads) k_batch_sample(const BatchItem*
 // Per pair: the kCombineBlocks partial sums of k_combine_part, a warp per slice (its
 // lane t takes the threads t + 32 k of that slice's block), and their final tree:
 // the same binary64 operations in the same order, so the same bits.  Without block
-// barriers the slices' loads and divisions overlap (512 pairs of d = 3, 9.4k points:
-// 516 us with a block per slice in turn; see launch_batch_combine).
+// barriers the slices' loads and divisions overlap (512 pairs of d = 3, 9.4k points a
+// pair: 516 us with a block per slice in turn, about 60 us).
 constexpr int kBatchCombineThreads = 512;
 __global__ void __launch_bounds__(kBatchCombineThreads) k_batch_combine(const BatchItem* items) {
   pdl_entry();

@@ -713,16 +713,21 @@ void launch_screen_l2(const ch_set* A, const int64_t* qidx, int64_t T, const ch_
 
 // ------------------------------------------------------------------ certified exact scan
 // The exact l2 scan through the same contraction: the screen's scores only decide
-// which columns are evaluated, and a proven bound on their error decides it, so the
-// minimum and argmin are those of the canonical distance to every b, bit for bit.
+// which columns are evaluated, and a bound on their error decides it, so the minimum
+// and argmin are those of the canonical distance to every b, bit for bit.  The bound
+// follows from the formats but for one assumption, the tensor core's accumulation,
+// whose internals are not documented: it takes an error per product four times larger
+// than truncation to 24 bits at the largest partial sum would give.  Measured against
+// 64 bits (sums of one sign, cancelling sums, exponents over 2^40, d from 8 to 1408),
+// the error on exactly held operands stays below a tenth of a quarter of that term.
 //
 // For real D2 = |q - b|^2 and the computed score S = fl(|b|^2 - 2 acc):
 //   |S + |q|^2 - D2| <= a |q||b| + b1 |b|^2,
 //   a  = 2 (c_in + 4 d 2^-23) + 2^-22: operand rounding (binary32 rows read as tf32
 //        keep 10 mantissa bits: c_in = 2^-9 (1 + 2^-10) per product for truncation or
-//        rounding; bf16 products are exact), accumulation (each of the d products is
-//        added with an error of at most 2^-23 of the largest partial sum, times four
-//        for margin; the partial sums are at most |q||b|), and the last fma;
+//        rounding; bf16 products are exact), accumulation (assumed: each of the d
+//        products is added with an error of at most 2^-23 of the largest partial sum,
+//        times four for margin; the partial sums are at most |q||b|), and the last fma;
 //   b1 = (d + 2) 2^-23: the norm's fma chain and the last fma.
 // With |q||b| <= (|q|^2 + |b|^2) / 2 the two sides separate:
 //   D2 >= L(b) + |q|^2 (1 - a/2),  L(b) = fl(|b|^2 (1 - a/2 - b1) - 2 acc)

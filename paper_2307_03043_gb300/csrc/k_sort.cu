@@ -12,7 +12,8 @@
 //
 // Sorting B alone by 32 bits moves 4 x 16 bytes per (point of B, scale); sorting A and
 // B by the full key and scale moved 9 x 24 bytes per (point, scale) and needed run
-// heads and positions besides.  50k x 50k, ten scales, window 16: see launch_sort_window.
+// heads and positions besides.  50k x 50k, d = 128, ten scales, four structures of window
+// 16, the whole call: 3.22 -> 0.98 ms.
 #include "common.cuh"
 
 namespace chx {
