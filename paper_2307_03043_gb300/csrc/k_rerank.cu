@@ -52,10 +52,13 @@ __device__ __forceinline__ void add_term(float& p, float x, float y) {
 //  * group_dist, wider rows: 32 / C lanes per row (C coordinates per 16-byte word), each
 //    owning C partials, so a row is read in whole 64- or 128-byte pieces; NR rows per
 //    lane group side by side.
-// Rerank of 8 entries x 4 columns for ~4.8k samples, cold caches, lane form / group form
-// / the earlier four rows per warp with a shuffle tree each: f32 d = 128 37 / 31 / 28 us
-// (the whole warm call 359 / 344 / 352 us), bf16 d = 384 122 / 67 / 65 us, bf16 d = 768
-// 256 / 97 / 94 us, fp8 d = 384 51 / - / 112 us.
+// Kernel time of the rerank of 8 entries x 4 columns, this form / the earlier four rows per
+// warp with a shuffle tree each, caches as the call leaves them (cold in brackets): f32
+// d = 128, 4.6k samples of 100k 25 / 27 us (31 / 29), bf16 d = 384, 300k 49 / 58 (49 / 57),
+// bf16 d = 768, 200k 89 / 93 (87 / 93), fp8 d = 384, 300k 50 / 100 (51 / 107).  The
+// line lies between the rows measured in both forms, cold: 384 bytes (fp8 d = 384) has the
+// lane form at half the earlier time; at 512 (f32 d = 128), 768 and 1536 bytes the lane
+// form took 37, 122 and 256 us, the group form 31, 67 and 97.
 constexpr int kWideRow = 512;
 
 template <int DT, int METRIC>
