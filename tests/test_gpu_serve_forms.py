@@ -90,13 +90,15 @@ def test_a_full_set_of_plain_footprints_runs_side_by_side(ctx, data, kind):
             alone[k] = s.wait(s.submit(_params(kind, k))[1])
     with _Server(ctx, data, SLOTS * plain, fault="slow") as s:
         s.wait(s.submit(_params(kind))[1])  # the pool and the contexts are warm
-        t0 = time.perf_counter()
-        ts = [s.submit(_params(kind, k))[1] for k in range(SLOTS)]
-        got = [s.wait(t) for t in ts]
-        wall = time.perf_counter() - t0
+        wall = []
+        for _ in range(4):
+            t0 = time.perf_counter()
+            ts = [s.submit(_params(kind, k))[1] for k in range(SLOTS)]
+            got = [s.wait(t) for t in ts]
+            wall.append(time.perf_counter() - t0)
+            assert got == [alone[k] for k in range(SLOTS)]
         assert s.peak() <= SLOTS * plain
-    assert got == [alone[k] for k in range(SLOTS)]
-    assert wall < 0.095, wall  # two in a row: 100 ms at least
+    assert min(wall) < 0.095, wall  # two in a row: 100 ms at least
 
 
 def test_a_wide_budget_admits_the_faster_form(ctx, data):
