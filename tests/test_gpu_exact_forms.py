@@ -173,3 +173,17 @@ def test_certified_brute_force_over_slices_of_small_rows(ctx):
     assert np.array_equal(mins.cpu().numpy(), mo) and abs(v / vo - 1) < 1e-12
     for s in (sA, sB):
         ch.ch_set_destroy(s)
+
+
+def test_more_listed_samples_than_the_kernel_writes_out(ctx):
+    """Past 65,536 samples the listed minima are written by a launch of their own."""
+    A, B = workloads.gaussian_mixture(70001, 601, 8, 9, clusters=6)
+    A, B = A + np.float32(1000), B + np.float32(1000)
+    sA, keepA, _ = _make(ctx, A, ch.CH_F32)
+    sB, keepB, _ = _make(ctx, B, ch.CH_F32)
+    mins = torch.zeros(70001, device="cuda")
+    v = ch.ch_exact(ctx, sA, sB, ch.CH_L2, 0, mins)
+    vo, mo = oracle.exact_canonical(A, B, ch.CH_L2)
+    assert np.array_equal(mins.cpu().numpy(), mo) and abs(v / vo - 1) < 1e-12
+    for s in (sA, sB):
+        ch.ch_set_destroy(s)
